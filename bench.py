@@ -887,26 +887,23 @@ def measured_traffic(record, src_path):
 
 def roofline_streamed(mape, wl, inst, starts, stream, prec, reps=2):
     """The streamed extraction of the large workload, timed live: `reps` calls
-    of mape_extract (T steps, the workload's starts and period) with the
-    library's per-launch CUDA events on the launches' streams.  A step is the
-    forward pass (reads z, writes sign(Bm z): (4 d + 2 R) bytes per start) and
-    the gradient + Adam pass (reads sign(Bm z) and reads and writes z, m, v:
-    (24 d + 2 R) bytes per start); the tiles run as two halves on two
-    streams, so that one half's forward pass overlaps the other's gradient
-    pass.  The unit of the roofline is therefore the step, both kernels
-    together: (28 d + 4 R) P bytes per step over the step's time (the call's
-    time over T, which includes packing z, m, v once per call).  The bound is
-    HBM bandwidth: the state (1.26 GB) is far larger than L2 and is streamed
-    every step.  The per-kernel launch durations are reported beside it; they
-    overlap in time."""
+    of mape_extract (T steps, the workload's starts and period).  A step reads
+    and writes the FP32 state z, m, v of every start and moves its operands of
+    z and signs; counted as (28 d + 4 R) P bytes (the state once in and out, z
+    once more, sign(Bm z) out and in) over the step's time (the call's time
+    over T, which includes turning z, m, v once per call).  The bound is HBM
+    bandwidth: the state (1.26 GB) is far larger than L2 and is streamed every
+    step.  Beside it, the launches of the step-by-step kernels (those of a
+    general B, which launch timing makes every call run)."""
     import numpy as np
     peaks, src = measured_peaks()
     P, T, d = wl["P"], wl["T"], inst.d
     R = inst.n - d
     host = tuple(None if a is None else a.cpu().numpy() for a in starts)
+    times, counts = time_extract_kernel(mape, inst, host, P, T, prec, stream, reps, period=wl["period"])
     mape.launch_timing(True)
     try:
-        times, counts = time_extract_kernel(mape, inst, host, P, T, prec, stream, reps, period=wl["period"])
+        stepwise, _ = time_extract_kernel(mape, inst, host, P, T, prec, stream, reps, period=wl["period"])
         per = mape.launch_timing_read()
     finally:
         mape.launch_timing(False)
@@ -925,19 +922,19 @@ def roofline_streamed(mape, wl, inst, starts, stream, prec, reps=2):
         kernels[name] = {"ms_per_launch": ms / max(n, 1), "launches_per_step": launches_per_step,
                          "bytes_per_launch": b, "achieved": b / (ms / max(n, 1) / 1e3) / 1e9,
                          "frac_while_overlapped": b / (ms / max(n, 1) / 1e3) / 1e9 / peak}
-    src_path = os.path.join(ROOT, "paper_2412_13576_gb300", "csrc", "extract_stream.cu")
-    return {"bound": "hbm", "kernel": "streamed step: stream_fwd_kernel and stream_grad_kernel, tile halves on two streams",
+    src_path = os.path.join(ROOT, "paper_2412_13576_gb300", "csrc", "extract_cluster.cu")
+    return {"bound": "hbm", "kernel": "cluster_kernel (all T steps in one launch), per step",
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": measured_traffic(STREAM_TRAFFIC, src_path), "ms_per_step": step_ms, "bytes_per_step": step_bytes,
             "peak_source": f"{src} HBM copy rate (MEASURED_PEAKS.json hbm_gbs)",
-            "kernels": kernels,
+            "step_by_step": {"ms_per_step": statistics.median(stepwise) / T, "kernels": kernels},
             "collect_ms_per_launch": per["stream_collect"][0] / max(per["stream_collect"][1], 1),
             "candidates_per_call": int(np.median(counts)),
             "note": "one step = forward + gradient (+ collection every period-th step) for P = 65536 starts, 28 d + 4 R "
                     "bytes per start; step time = CUDA-event time of a T = 1000 call / T (the call also packs z, m, v "
-                    "once); kernel launch durations from events the library records around each launch on its "
-                    "stream; traffic = ncu dram read+write bytes of one step (both kernels), null unless taken on "
-                    "this source"}
+                    "once); step_by_step: the kernels that launch timing makes the call run, from events the library "
+                    "records around each launch; traffic = ncu dram read+write bytes of one step, null unless taken "
+                    "on this source"}
 
 
 def roofline_resident(mape, wl, inst, G0, stream, reps=3):

@@ -90,9 +90,12 @@ extern "C" {
  *   resident: one persistent fused kernel for all T steps, B and the tile's
  *             z, m, v on chip; for tiles that fit (rows of B through the MMA
  *             and d at most 256, the operands within shared memory);
- *   streamed: three kernels per step (forward + map, collect, gradient +
- *             Adam) over tiles of 128 starts, with B and the state streamed
- *             through shared memory by bulk copies; any n, d <= 4096.
+ *   streamed: tiles of 128 starts with B and the state streamed through
+ *             shared memory by bulk copies; any n, d <= 4096.  An
+ *             identity-topped B runs in one launch for all T steps, a cluster
+ *             of thread blocks per tile; a general B (and every B while
+ *             mape_launch_timing is on) in three kernels per step (forward +
+ *             map, collect, gradient + Adam).  Both give the same bits.
  * The resident kernel is chosen when it fits; OR-ing MAPE_PREC_STREAMED into
  * the precision forces the streamed one. */
 #define MAPE_PREC_STREAMED 0x100
@@ -234,9 +237,9 @@ int mape_extract(const mape_extract_args* args, void* stream);
  * counter, flags and workspace of mape_extract_workspace_bytes), all with the
  * same t0, T, period and BF16 precision.  The calls that fit the resident
  * kernel run as one persistent launch per kernel variant (identity-topped or
- * general B, state in TMEM or not) over all their tiles; the others run the
- * streamed kernels with three launches per step covering all of them; all of
- * it is captured into one CUDA graph and launched (not on the legacy default
+ * general B, state in TMEM or not) over all their tiles; of the others, those
+ * with an identity-topped B run as one launch per cluster size over all their
+ * tiles, a general B with three launches per step; all of it is captured into one CUDA graph and launched (not on the legacy default
  * stream, which is not capturable: there the kernels are launched directly).
  * Each call's results are identical to its own mape_extract.  `workspace`
  * holds the batch's tables (mape_extract_batch_workspace_bytes).
@@ -853,7 +856,8 @@ void mape_server_destroy(mape_server_h s);
  * of launches since timing was switched on (or last read: reading clears the
  * pending pairs, not the sums).  mape_launch_timing(enable) switches it and
  * clears everything.  The events add a little time around each launch, so
- * time a region either with or without it. */
+ * time a region either with or without it.  While it is on, streamed calls run
+ * step by step for every B, since these kinds are launches of one step. */
 #define MAPE_TIMED_STREAM_FWD     0   /* streamed forward + map kernel       */
 #define MAPE_TIMED_STREAM_COLLECT 1   /* streamed collection kernel          */
 #define MAPE_TIMED_STREAM_GRAD    2   /* streamed gradient + Adam kernel     */

@@ -183,6 +183,8 @@ size_t tune_scratch_bytes(int32_t n, int32_t d, int32_t P) {
 
 int run_choice(const mape_extract_args* a, cudaStream_t st, const mape_tune_info& c) {
   if (c.path == 0) return mape_detail::extract_tc(a, st);
+  // the widest blocks stand for the default implementation
+  if (c.path == 1 && c.wF == 256 && c.wG == 256) return mape_detail::extract_stream(a, st, mape_detail::kFwdDense);
   return mape_detail::extract_stream_widths(a, st, c.wF, c.wG,
                                             c.path == 2 ? mape_detail::kFwdSparse : mape_detail::kFwdDense);
 }
@@ -292,7 +294,11 @@ extern "C" size_t mape_extract_workspace_bytes(int32_t n, int32_t d, int32_t P, 
   const int32_t base = precision & MAPE_PREC_MASK;
   if (base == MAPE_PREC_FP32) return mape_detail::extract_fp32_workspace(n, d, P);
   if (base == MAPE_PREC_SPARSE) return mape_detail::extract_sparse_workspace(n, d, P);
-  if (base == MAPE_PREC_FP8) return mape_detail::extract_stream_workspace(n, d, P);
+  const size_t cl = mape_detail::extract_cluster_workspace(n, d, P, base);
+  if (base == MAPE_PREC_FP8) {
+    const size_t w = mape_detail::extract_stream_workspace(n, d, P);
+    return w && cl > w ? cl : w;
+  }
   // the streamed path also serves a general B of a shape whose resident tile
   // fits only when B is identity-topped, so its workspace is always included
   size_t w = mape_detail::extract_stream_workspace(n, d, P);
@@ -300,6 +306,7 @@ extern "C" size_t mape_extract_workspace_bytes(int32_t n, int32_t d, int32_t P, 
     const size_t t = mape_detail::extract_tc_workspace(n, d, P, base);
     if (t > w) w = t;
   }
+  if (w && cl > w) w = cl;
   return w;
 }
 

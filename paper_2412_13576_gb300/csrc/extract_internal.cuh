@@ -39,6 +39,18 @@ int extract_stream(const mape_extract_args* a, cudaStream_t st, int fwd_mode);
 // the same with the forward and gradient N-block widths chosen (64..256, multiples of 64)
 int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, int wG, int fwd_mode);
 
+// the same for an identity-topped B in one launch of tile clusters
+// (extract_cluster.cu); *general = true, and nothing done, for another B
+size_t extract_cluster_workspace(int32_t n, int32_t d, int32_t P, int32_t precision);
+int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general);
+// and for a batch of such calls (same T, t0, period, precision)
+struct ClBatch;
+size_t extract_cluster_batch_workspace(const mape_extract_args* const* items, int count);
+int extract_cluster_batch_prepare(const mape_extract_args* const* items, int count, void* ws, size_t ws_bytes,
+                                  cudaStream_t st, ClBatch** out);
+int extract_cluster_batch_enqueue(const ClBatch* plan, cudaStream_t st);
+void extract_cluster_batch_free(ClBatch* plan);
+
 // Batches of calls on the streamed kernels: three launches per step for all
 // calls of one basis kind.
 struct StBatch;

@@ -15,8 +15,7 @@
 
 namespace mape_tc {
 
-constexpr uint64_t kWaitNs = 2000000000ull;  // 2 s of the global timer
-constexpr uint32_t kWaitLimit = 1u << 22;
+constexpr long long kWaitCycles = 4000000000ll;  // of the SM clock: 2 s at its 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -165,20 +164,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// wait for the phase of the given parity, bounded in time and iterations;
-// returns false on time-out
+// wait for the phase of the given parity, bounded in time; returns false on
+// time-out.  The bound is counted on the SM clock, read only once a first try
+// failed: a read of the global timer costs some hundred cycles, and with one
+// per wait the waits of a chunked pipeline took most of its time.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
-  const uint64_t t0 = global_ns();
-  for (uint32_t i = 0; i < kWaitLimit; ++i) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  do {
     if (mbar_try_wait(bar, parity)) return true;
-    if (global_ns() - t0 > kWaitNs) return false;
-  }
+  } while (clock64() - t0 < kWaitCycles);
   return false;
 }
 
@@ -221,6 +216,56 @@ constexpr uint32_t kChunkLbo = 128;
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// The issuing instructions for a converged warp, performed by the lane whose
+// `lead` is nonzero (elect_lead): the code around them stays warp-uniform, so
+// that descriptors, addresses and counts live in uniform registers.  Issued
+// from a branch of one thread, an MMA costs about 110 cycles of moves into
+// them, this way 40 to 60.
+__device__ __forceinline__ uint32_t elect_lead() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
+}
+// a, b: the low words of the operands' descriptors (address and LBO), hi: their
+// common high word (SBO, version)
+__device__ __forceinline__ void mma_bf16_if(uint32_t lead, uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t hi,
+                                            uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc), "r"(lead));
+}
+__device__ __forceinline__ void mma_e4m3_if(uint32_t lead, uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t hi,
+                                            uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc), "r"(lead));
+}
+__device__ __forceinline__ void mma_commit_if(uint32_t lead, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+      "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_if(uint32_t lead, uint32_t bar, uint32_t bytes) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
+      " @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(bar),
+      "r"(bytes), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void bulk_g2s_if(uint32_t lead, uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %4, 0;\n"
+      " @q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}\n" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar), "r"(lead)
+      : "memory");
 }
 
 }  // namespace mape_tc
