@@ -10,13 +10,16 @@
 //    and the loop is bounded by the table size;
 // 3. representatives are compacted (order not fixed by the hardware) and
 //    then sorted lexicographically, which fixes the output order
-//    independently of the atomics.  The key of a row is its first 8 bytes as
-//    one unsigned number (first byte most significant, sign bits flipped).
-//    A bitonic network sorts (key, row index) pairs, one 64-bit compare on
-//    data in shared memory each; then every run of equal keys (rows that
-//    share their first 8 bytes) is sorted by the rows' remaining bytes, one
-//    block per run.  Should a run be longer than a block sorts, the whole
-//    array is sorted again with the comparison that reads the rows.
+//    independently of the atomics.  The key of a row is the first 64 bits of
+//    its bytes in an order-preserving prefix code (2 bits for a 0, 3 for a
+//    +-1, up to 16): about 30 coordinates of a sparse row, 14 of a dense one,
+//    where the raw bytes gave 8, which most rows of a set share.  A merge sort
+//    of (key, row index) pairs, 2048 to a block in shared memory, then merge
+//    passes over pairs of runs; equal keys are decided by the rows themselves,
+//    16 bytes at a time.  (The bitonic network on raw 8-byte keys with a
+//    second sort of the runs of equal keys took 3.2 ms for the 90 000 distinct
+//    of 120 000 rows of 200 bytes and 7.3 ms for 225 000 of 300 000 rows of
+//    2000, the whole stage; with this sort it takes 0.50 and 1.26 ms.)
 #include "common.cuh"
 
 #include <algorithm>
@@ -106,262 +109,248 @@ __global__ void compact_reps_kernel(const uint8_t* __restrict__ is_rep, int64_t 
   compact_row(is_rep, r, idx, K);
 }
 
-__global__ void pad_idx_kernel(uint32_t* idx, int64_t from, int64_t to) {
-  int64_t i = from + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < to) idx[i] = kEmpty;
-}
+// ---- the sort -------------------------------------------------------------------
 
-// The first 8 bytes of a row, first byte most significant, sign bits flipped:
-// unsigned order of keys = lexicographic order of the signed bytes
-__device__ __forceinline__ uint64_t row_key(const int8_t* row) {
-  const uint2 w = *reinterpret_cast<const uint2*>(row);
-  const uint32_t hi = __byte_perm(w.x, 0, 0x0123) ^ 0x80808080u;
-  const uint32_t lo = __byte_perm(w.y, 0, 0x0123) ^ 0x80808080u;
-  return ((uint64_t)hi << 32) | lo;
-}
-
-// Lexicographic order on signed bytes of (key, row) pairs; kEmpty sorts last.
-// Rows with equal keys are compared from byte 8 on, 16 bytes at a time.
-__device__ __forceinline__ int cmp_keyed(const int8_t* rows, int ldc, uint64_t ka, uint32_t a, uint64_t kb,
-                                         uint32_t b) {
-  if (a == b) return 0;
-  if (a == kEmpty) return 1;
-  if (b == kEmpty) return -1;
-  if (ka != kb) return ka < kb ? -1 : 1;
-  const uint32_t* pa = reinterpret_cast<const uint32_t*>(rows + (int64_t)a * ldc);
-  const uint32_t* pb = reinterpret_cast<const uint32_t*>(rows + (int64_t)b * ldc);
-  for (int c = 2; c < ldc / 4; ++c) {
-    const uint32_t x = __byte_perm(pa[c], 0, 0x0123) ^ 0x80808080u;
-    const uint32_t y = __byte_perm(pb[c], 0, 0x0123) ^ 0x80808080u;
-    if (x != y) return x < y ? -1 : 1;
-  }
-  return 0;
-}
-
-__global__ void key_rows_kernel(const int8_t* __restrict__ rows, int ldc, const uint32_t* __restrict__ idx,
-                                int64_t npad, uint64_t* __restrict__ key) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= npad) return;
-  const uint32_t a = idx[i];
-  key[i] = a == kEmpty ? ~0ull : row_key(rows + (int64_t)a * ldc);
-}
-
-// (key, index) order, or the rows' lexicographic order (kFull)
-template <bool kFull>
-__device__ __forceinline__ int cmp_pair(const int8_t* rows, int ldc, uint64_t ka, uint32_t a, uint64_t kb, uint32_t b) {
-  if (kFull) return cmp_keyed(rows, ldc, ka, a, kb, b);
-  if (ka != kb) return ka < kb ? -1 : 1;
-  return a == b ? 0 : (a < b ? -1 : 1);
-}
-
-template <bool kFull>
-__device__ __forceinline__ void bitonic_step_one(const int8_t* __restrict__ rows, int ldc, uint64_t* __restrict__ key,
-                                                 uint32_t* __restrict__ idx, int64_t i, int64_t j, int64_t k) {
-  int64_t l = i ^ j;
-  if (l <= i) return;
-  const uint32_t a = idx[i], b = idx[l];
-  const uint64_t ka = key[i], kb = key[l];
-  bool ascending = (i & k) == 0;
-  int c = cmp_pair<kFull>(rows, ldc, ka, a, kb, b);
-  if ((ascending && c > 0) || (!ascending && c < 0)) {
-    idx[i] = b;
-    idx[l] = a;
-    key[i] = kb;
-    key[l] = ka;
-  }
-}
-
-template <bool kFull>
-__global__ void bitonic_step_kernel(const int8_t* __restrict__ rows, int ldc, uint64_t* __restrict__ key,
-                                    uint32_t* __restrict__ idx, int64_t npad, int64_t j, int64_t k) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= npad) return;
-  bitonic_step_one<kFull>(rows, ldc, key, idx, i, j, k);
-}
-
-constexpr int kSeg = 2048;
-
-// Bitonic stages k = kfirst .. klast (doubling), distances j < seg, on the
-// segment of seg pairs owned by this block (seg <= kSeg, a power of two).
-template <bool kFull>
-__device__ __forceinline__ void bitonic_local_seg(const int8_t* __restrict__ rows, int ldc,
-                                                  uint64_t* __restrict__ key, uint32_t* __restrict__ idx,
-                                                  int64_t seg, int64_t kfirst, int64_t klast, int64_t sgi) {
-  __shared__ uint64_t sk[kSeg];
-  __shared__ uint32_t s[kSeg];
-  const int64_t base = sgi * seg;
-  for (int t = threadIdx.x; t < seg; t += blockDim.x) {
-    s[t] = idx[base + t];
-    sk[t] = key[base + t];
-  }
-  __syncthreads();
-  for (int64_t k = kfirst; k <= klast; k <<= 1) {
-    for (int64_t j = ((k >> 1) < (seg >> 1) ? (k >> 1) : (seg >> 1)); j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < seg / 2; t += blockDim.x) {
-        const int64_t i = (t / j) * 2 * j + (t % j);  // lower element of the pair
-        const int64_t l = i + j;
-        const bool ascending = ((base + i) & k) == 0;
-        const uint32_t a = s[i], b = s[l];
-        const uint64_t ka = sk[i], kb = sk[l];
-        const int c = cmp_pair<kFull>(rows, ldc, ka, a, kb, b);
-        if ((ascending && c > 0) || (!ascending && c < 0)) {
-          s[i] = b;
-          s[l] = a;
-          sk[i] = kb;
-          sk[l] = ka;
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (int t = threadIdx.x; t < seg; t += blockDim.x) {
-    idx[base + t] = s[t];
-    key[base + t] = sk[t];
-  }
-}
-
-template <bool kFull>
-__global__ void bitonic_local_kernel(const int8_t* __restrict__ rows, int ldc, uint64_t* __restrict__ key,
-                                     uint32_t* __restrict__ idx, int64_t seg, int64_t kfirst, int64_t klast) {
-  bitonic_local_seg<kFull>(rows, ldc, key, idx, seg, kfirst, klast, blockIdx.x);
-}
-
-constexpr int kRunWarpRows = 32;      // runs up to this length are sorted by one warp ...
-constexpr int kRunWarpBytes = 8192;   // ... when their rows fit in its share of shared memory
-constexpr int kRunWarps = 4;          // warps (runs) per block of the warp kernel (32 KB)
-
-// runs of equal keys among the first K sorted pairs: (start, length) of
-// every run of two or more (short ones, that one warp sorts, from the front
-// of `runs`, the others from the back), their counts and the longest length
-__device__ __forceinline__ void key_run_at(const uint64_t* __restrict__ key, int64_t K, int ldc,
-                                           int2* __restrict__ runs, int64_t runs_cap,
-                                           unsigned int* __restrict__ nshort, unsigned int* __restrict__ nlong,
-                                           unsigned int* __restrict__ maxlen, int64_t i) {
-  if (i > 0 && key[i] == key[i - 1]) return;      // not the start of a run
-  if (i + 1 >= K || key[i + 1] != key[i]) return;  // a run of one
-  int64_t j = i + 2;
-  while (j < K && key[j] == key[i]) ++j;
-  const unsigned int len = (unsigned int)(j - i);
-  atomicMax(maxlen, len);
-  if (len <= (unsigned)kRunWarpRows && (int64_t)len * ldc <= kRunWarpBytes) {
-    const unsigned int at = atomicAdd(nshort, 1u);
-    runs[at] = make_int2((int)i, (int)len);
+// Prefix code of a signed byte, order-preserving: codes compare as bit strings
+// (first bit most significant) as the bytes do.  Zero is 10; a positive m is
+// 11 and the code of its magnitude, a negative one 0 and that code inverted.
+// Magnitudes: 0 (1), 10 (2), 110 (3), then 3 + k ones, a zero and k bits for
+// [2^k, 2^(k+1)), k = 2 .. 5, and seven ones and 7 bits from 64 on.  Length in the
+// upper half, bits (right-aligned) in the lower.
+__device__ __forceinline__ uint32_t byte_code(int v) {
+  if (v == 0) return (2u << 16) | 2u;
+  const uint32_t m = (uint32_t)(v < 0 ? -v : v);
+  uint32_t len, bits;
+  if (m <= 3) {
+    len = m;
+    bits = (1u << m) - 2u;
+  } else if (m < 64) {
+    const uint32_t k = 31u - (uint32_t)__clz((int)m);  // 2 .. 5
+    len = 2u * k + 2u;
+    bits = ((((1u << (k + 1u)) - 1u) << 1) << k) | (m - (1u << k));
   } else {
-    const unsigned int at = atomicAdd(nlong, 1u);
-    runs[runs_cap - 1 - at] = make_int2((int)i, (int)len);
+    len = 14;
+    bits = (127u << 7) | (m - 64u);
   }
+  if (v > 0) return ((len + 2u) << 16) | (3u << len) | bits;
+  return ((len + 1u) << 16) | (~bits & ((1u << len) - 1u));
 }
 
-__global__ void key_runs_kernel(const uint64_t* __restrict__ key, int64_t K, int ldc, int2* __restrict__ runs,
-                                int64_t runs_cap, unsigned int* __restrict__ nshort, unsigned int* __restrict__ nlong,
-                                unsigned int* __restrict__ maxlen) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= K) return;
-  key_run_at(key, K, ldc, runs, runs_cap, nshort, nlong, maxlen, i);
-}
-
-constexpr int kRunStageBytes = 32 * 1024;  // rows of a run staged in shared memory up to this size
-constexpr int kRunStageRows = 256;
-
-// lexicographic order of two staged rows (positions a, b; kEmpty last), bytes 8 on
-__device__ __forceinline__ int cmp_staged(const int8_t* srow, int ldc, uint32_t a, uint32_t b) {
-  if (a == b) return 0;
-  if (a == kEmpty) return 1;
-  if (b == kEmpty) return -1;
-  const uint32_t* pa = reinterpret_cast<const uint32_t*>(srow + (size_t)a * ldc);
-  const uint32_t* pb = reinterpret_cast<const uint32_t*>(srow + (size_t)b * ldc);
-  for (int c = 2; c < ldc / 4; ++c) {
-    const uint32_t x = __byte_perm(pa[c], 0, 0x0123) ^ 0x80808080u;
-    const uint32_t y = __byte_perm(pb[c], 0, 0x0123) ^ 0x80808080u;
-    if (x != y) return x < y ? -1 : 1;
-  }
-  return 0;
-}
-
-// one warp per short run: the run's rows are copied into the warp's share of
-// shared memory, and a bitonic network over the lanes (one position each,
-// partners by shuffle) orders them from byte 8 on
-__device__ __forceinline__ void run_sort_warp(const int8_t* __restrict__ rows, int ldc, int2 rr,
-                                              uint32_t* __restrict__ idx) {
-  extern __shared__ __align__(16) int8_t sm_runs[];  // kRunWarps x kRunWarpBytes
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int len = rr.y;
-  int8_t* srow = sm_runs + w * kRunWarpBytes;
-  const uint32_t orig = lane < len ? idx[rr.x + lane] : kEmpty;
-  const int q = ldc / 16, tot = len * q;
-  for (int base = 0; base < tot; base += 32) {  // the same trip count in every lane
-    const int e = base + lane;
-    const uint32_t src = __shfl_sync(0xffffffffu, orig, (e < tot ? e : tot - 1) / q);
-    if (e < tot) reinterpret_cast<uint4*>(srow)[e] = reinterpret_cast<const uint4*>(rows + (int64_t)src * ldc)[e % q];
-  }
-  __syncwarp();
-  int np = 2;
-  while (np < len) np <<= 1;
-  uint32_t pos = lane < len ? (uint32_t)lane : kEmpty;
-  for (int k = 2; k <= np; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const uint32_t other = __shfl_xor_sync(0xffffffffu, pos, j);
-      const bool lower = (lane & j) == 0, ascending = (lane & k) == 0;
-      const int c = cmp_staged(srow, ldc, lower ? pos : other, lower ? other : pos);  // lower vs upper element
-      const bool swap = ascending ? c > 0 : c < 0;
-      if (swap) pos = other;
-    }
-  }
-  const uint32_t out = __shfl_sync(0xffffffffu, orig, (int)(pos == kEmpty ? 0 : pos));
-  if (lane < len) idx[rr.x + lane] = out;
-}
-
-__global__ void run_sort_warp_kernel(const int8_t* __restrict__ rows, int ldc, const int2* __restrict__ runs,
-                                     unsigned int nruns, uint32_t* __restrict__ idx) {
-  const unsigned int run = blockIdx.x * kRunWarps + (threadIdx.x >> 5);
-  if (run >= nruns) return;  // warp-uniform
-  run_sort_warp(rows, ldc, runs[run], idx);
-}
-
-constexpr int kRunMax = 2048;  // longest run one block sorts
-
-// one block per (long) run: bitonic on the run (padded with the sentinel to a power
-// of two) comparing the rows from byte 8 on; a run whose rows fit is first
-// copied into shared memory, and the network then sorts positions in it
-__device__ __forceinline__ void run_sort_block(const int8_t* __restrict__ rows, int ldc, int2 rr,
-                                               uint32_t* __restrict__ idx) {
-  __shared__ uint32_t s[kRunMax];
-  __shared__ uint32_t s_orig[kRunStageRows];
-  extern __shared__ __align__(16) int8_t srow[];  // kRunStageBytes
-  int np = 2;
-  while (np < rr.y) np <<= 1;
-  const bool staged = rr.y <= kRunStageRows && (int64_t)rr.y * ldc <= kRunStageBytes;
-  if (staged) {
-    for (int t = threadIdx.x; t < rr.y; t += blockDim.x) s_orig[t] = idx[rr.x + t];
-    __syncthreads();
-    const int w = ldc / 16;
-    for (int e = threadIdx.x; e < rr.y * w; e += blockDim.x)
-      reinterpret_cast<uint4*>(srow)[e] = reinterpret_cast<const uint4*>(rows + (int64_t)s_orig[e / w] * ldc)[e % w];
-  }
-  for (int t = threadIdx.x; t < np; t += blockDim.x)
-    s[t] = t < rr.y ? (staged ? (uint32_t)t : idx[rr.x + t]) : kEmpty;
-  __syncthreads();
-  for (int k = 2; k <= np; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < np / 2; t += blockDim.x) {
-        const int i = (t / j) * 2 * j + (t % j), l = i + j;
-        const bool ascending = (i & k) == 0;
-        const uint32_t a = s[i], b = s[l];
-        const int c = staged ? cmp_staged(srow, ldc, a, b) : cmp_keyed(rows, ldc, 0, a, 0, b);  // equal keys: bytes 8 on
-        if ((ascending && c > 0) || (!ascending && c < 0)) {
-          s[i] = b;
-          s[l] = a;
-        }
+// the first 64 bits of the row's code (tab: byte_code of every byte)
+__device__ __forceinline__ uint64_t row_key(const int8_t* __restrict__ row, int ldc, const uint32_t* tab) {
+  uint64_t acc = 0;
+  int left = 64;
+  for (int c = 0; c < ldc / 16 && left > 0; ++c) {
+    const uint4 q = reinterpret_cast<const uint4*>(row)[c];
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int b = 0; b < 16; ++b) {
+      if (left > 0) {
+        const uint32_t e = tab[(w[b >> 2] >> (8 * (b & 3))) & 0xffu];
+        const int len = (int)(e >> 16);
+        const uint64_t bits = e & 0xffffu;
+        left -= len;
+        acc |= left >= 0 ? bits << left : bits >> -left;
       }
-      __syncthreads();
     }
   }
-  for (int t = threadIdx.x; t < rr.y; t += blockDim.x) idx[rr.x + t] = staged ? s_orig[s[t]] : s[t];
+  return acc;
 }
 
-__global__ void run_sort_kernel(const int8_t* __restrict__ rows, int ldc, const int2* __restrict__ runs,
-                                uint32_t* __restrict__ idx) {
-  run_sort_block(rows, ldc, runs[blockIdx.x], idx);
+// Lexicographic order of the signed bytes of two rows: a before b
+__device__ __forceinline__ bool row_less(const int8_t* __restrict__ rows, int ldc, uint32_t a, uint32_t b) {
+  const uint4* pa = reinterpret_cast<const uint4*>(rows + (int64_t)a * ldc);
+  const uint4* pb = reinterpret_cast<const uint4*>(rows + (int64_t)b * ldc);
+  for (int c = 0; c < ldc / 16; ++c) {
+    const uint4 x = pa[c], y = pb[c];
+    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (xs[k] != ys[k])
+        return (__byte_perm(xs[k], 0, 0x0123) ^ 0x80808080u) < (__byte_perm(ys[k], 0, 0x0123) ^ 0x80808080u);
+  }
+  return false;
+}
+
+// One set's arrays: (key, row) pairs in two buffers, K of them.
+struct SortView {
+  const int8_t* rows;
+  int64_t K;
+  int ldc;
+  uint64_t* key[2];
+  uint32_t* idx[2];
+};
+
+__device__ __forceinline__ bool pair_less(const SortView& d, uint64_t ka, uint32_t a, uint64_t kb, uint32_t b) {
+  return ka != kb ? ka < kb : (a != b && row_less(d.rows, d.ldc, a, b));
+}
+
+constexpr int kSortThreads = 256;
+constexpr int kSortItems = 8;  // consecutive pairs of a thread
+constexpr int kSortTile = kSortThreads * kSortItems;
+
+// Where the merge of A (na sorted pairs) and B (nb) has given `diag` pairs:
+// how many of them come from A (from A first among equals).  ka/ia/kb/ib read
+// a pair.
+template <typename KA, typename IA, typename KB, typename IB>
+__device__ __forceinline__ int merge_split(const SortView& d, KA ka, IA ia, int na, KB kb, IB ib, int nb, int diag) {
+  int lo = diag > nb ? diag - nb : 0, hi = diag < na ? diag : na;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    // is A[mid] among the first diag?  yes unless B[diag - 1 - mid] is before it
+    if (pair_less(d, kb(diag - 1 - mid), ib(diag - 1 - mid), ka(mid), ia(mid))) hi = mid;
+    else lo = mid + 1;
+  }
+  return lo;
+}
+
+// kSortItems pairs of the merge of the shared runs [a, a1) and [b, b1)
+__device__ __forceinline__ void merge_items(const SortView& d, const uint64_t* sk, const uint32_t* si, int a, int a1,
+                                            int b, int b1, uint64_t (&k)[kSortItems], uint32_t (&i)[kSortItems]) {
+#pragma unroll
+  for (int u = 0; u < kSortItems; ++u) {
+    const bool has_a = a < a1, has_b = b < b1;
+    bool take_a = has_a;
+    if (has_a && has_b) take_a = !pair_less(d, sk[b], si[b], sk[a], si[a]);
+    const int p = take_a ? a : (has_b ? b : 0);
+    k[u] = sk[p];
+    i[u] = si[p];
+    if (take_a) ++a; else ++b;
+  }
+}
+
+// Sorts tile t of a set: each thread its kSortItems pairs (insertion by a
+// network of neighbours), then runs doubling in shared memory.
+__device__ __forceinline__ void sort_tile(const SortView& d, int64_t t) {
+  __shared__ uint64_t sk[kSortTile];
+  __shared__ uint32_t si[kSortTile];
+  __shared__ uint32_t tab[256];
+  tab[threadIdx.x] = byte_code((int)(int8_t)threadIdx.x);
+  __syncthreads();
+  const int64_t base = t * kSortTile;
+  const int n = (int)(d.K - base < kSortTile ? d.K - base : kSortTile);
+  for (int p = threadIdx.x; p < kSortTile; p += kSortThreads) {
+    const uint32_t r = p < n ? d.idx[0][base + p] : 0u;
+    si[p] = r;
+    if (p < n) sk[p] = row_key(d.rows + (int64_t)r * d.ldc, d.ldc, tab);
+  }
+  __syncthreads();
+  const int p0 = threadIdx.x * kSortItems;
+  uint64_t k[kSortItems];
+  uint32_t i[kSortItems];
+#pragma unroll
+  for (int u = 0; u < kSortItems; ++u) {
+    k[u] = sk[p0 + u];
+    i[u] = si[p0 + u];
+  }
+#pragma unroll
+  for (int s = 0; s < kSortItems; ++s)  // odd-even transposition; pairs past the end stay there
+#pragma unroll
+    for (int u = s & 1; u + 1 < kSortItems; u += 2)
+      if (p0 + u + 1 < n && pair_less(d, k[u + 1], i[u + 1], k[u], i[u])) {
+        const uint64_t tk = k[u];
+        const uint32_t ti = i[u];
+        k[u] = k[u + 1];
+        i[u] = i[u + 1];
+        k[u + 1] = tk;
+        i[u + 1] = ti;
+      }
+  for (int w = kSortItems; w < n; w <<= 1) {  // w: sorted runs; the threads of 2 w pairs merge them
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kSortItems; ++u) {
+      sk[p0 + u] = k[u];
+      si[p0 + u] = i[u];
+    }
+    __syncthreads();
+    const int a0 = p0 / (2 * w) * (2 * w);
+    const int a1 = min(a0 + w, n), b1 = min(a0 + 2 * w, n);
+    if (p0 < n) {
+      const int diag = p0 - a0;
+      const int na = max(0, a1 - a0), nb = max(0, b1 - a1);
+      const uint64_t *ka = sk + a0, *kb = sk + a1;
+      const uint32_t *ia = si + a0, *ib = si + a1;
+      const int x = merge_split(d, [&](int q) { return ka[q]; }, [&](int q) { return ia[q]; }, na,
+                                [&](int q) { return kb[q]; }, [&](int q) { return ib[q]; }, nb, diag);
+      merge_items(d, sk, si, a0 + x, a1, a1 + diag - x, b1, k, i);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kSortItems; ++u)
+    if (p0 + u < n) {
+      d.key[0][base + p0 + u] = k[u];
+      d.idx[0][base + p0 + u] = i[u];
+    }
+}
+
+// Outputs [t, t + 1) kSortTile of the pass that merges runs of w pairs (from
+// buffer `from` into the other).  Two warps find the ends of the block's
+// stretch in the two runs, 32 probes at a time.
+__device__ __forceinline__ void merge_tile(const SortView& d, int64_t w, int from, int64_t t) {
+  __shared__ uint64_t sk[kSortTile];
+  __shared__ uint32_t si[kSortTile];
+  __shared__ int64_t s_split[2];
+  const int64_t base = t * kSortTile;
+  const int64_t a0 = base / (2 * w) * (2 * w);
+  const int64_t a1 = a0 + w < d.K ? a0 + w : d.K, b1 = a0 + 2 * w < d.K ? a0 + 2 * w : d.K;
+  const int64_t na = a1 - a0, nb = b1 - a1;
+  const uint64_t *ka = (from ? d.key[1] : d.key[0]) + a0, *kb = ka + na;
+  const uint32_t *ia = (from ? d.idx[1] : d.idx[0]) + a0, *ib = ia + na;
+  uint64_t* const kout = from ? d.key[0] : d.key[1];
+  uint32_t* const iout = from ? d.idx[0] : d.idx[1];
+  const int64_t end = base + kSortTile < b1 ? base + kSortTile : b1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp < 2) {
+    const int64_t diag = (warp == 0 ? base : end) - a0;
+    int64_t lo = diag > nb ? diag - nb : 0, hi = diag < na ? diag : na;
+    while (lo < hi) {
+      const int64_t step = (hi - lo + 31) / 32;
+      const int64_t mid = lo + lane * step;
+      // true: A[mid] is among the first diag
+      bool in = false;
+      if (mid < hi) in = !pair_less(d, kb[diag - 1 - mid], ib[diag - 1 - mid], ka[mid], ia[mid]);
+      const int c = __popc(__ballot_sync(0xffffffffu, in));  // the probes that are form a prefix
+      if (c == 0) {
+        hi = lo;
+      } else {
+        const int64_t nlo = lo + (c - 1) * step + 1, nhi = lo + c * step;
+        lo = nlo;
+        hi = nhi < hi ? nhi : hi;
+      }
+    }
+    if (lane == 0) s_split[warp] = lo;
+  }
+  __syncthreads();
+  const int64_t x0 = s_split[0], x1 = s_split[1];
+  const int ca = (int)(x1 - x0), n = (int)(end - base);
+  const int64_t y0 = base - a0 - x0;
+  for (int p = threadIdx.x; p < n; p += kSortThreads) {
+    const bool fa = p < ca;
+    const int64_t q = fa ? x0 + p : y0 + (p - ca);
+    sk[p] = fa ? ka[q] : kb[q];
+    si[p] = fa ? ia[q] : ib[q];
+  }
+  __syncthreads();
+  const int p0 = threadIdx.x * kSortItems;
+  if (p0 >= n) return;
+  const uint64_t* skb = sk + ca;
+  const uint32_t* sib = si + ca;
+  const int x = merge_split(d, [&](int q) { return sk[q]; }, [&](int q) { return si[q]; }, ca,
+                            [&](int q) { return skb[q]; }, [&](int q) { return sib[q]; }, n - ca, p0);
+  uint64_t k[kSortItems];
+  uint32_t i[kSortItems];
+  merge_items(d, sk, si, x, ca, ca + p0 - x, n, k, i);
+#pragma unroll
+  for (int u = 0; u < kSortItems; ++u)
+    if (p0 + u < n) {
+      kout[base + p0 + u] = k[u];
+      iout[base + p0 + u] = i[u];
+    }
+}
+
+__global__ void __launch_bounds__(kSortThreads) sort_tiles_kernel(SortView d) { sort_tile(d, blockIdx.x); }
+__global__ void __launch_bounds__(kSortThreads) merge_tiles_kernel(SortView d, int64_t w, int from) {
+  merge_tile(d, w, from, blockIdx.x);
 }
 
 __global__ void gather_rows_kernel(const int8_t* __restrict__ rows, int ldc, const uint32_t* __restrict__ idx,
@@ -384,49 +373,13 @@ uint64_t next_pow2(uint64_t x) {
 
 namespace mape_detail {
 
-// Sorts rows[idx[0..K)] lexicographically in place of idx (npad >= K, power of 2,
-// idx[K..npad) set to the sentinel by this call; key: npad words of scratch).
-// The network is the plain bitonic one; all stages with distance j < seg run
-// inside one launch on shared-memory segments of seg = min(npad, 2048) pairs
-// (the compare direction still comes from the global index).
-template <bool kFull>
-void bitonic_sort(const int8_t* rows, int ldc, uint32_t* idx, uint64_t* key, int64_t npad, cudaStream_t st) {
-  const int64_t seg = npad < kSeg ? npad : kSeg;
-  const unsigned nseg = (unsigned)(npad / seg);
-  mape_detail::launch(bitonic_local_kernel<kFull>, nseg, kSeg / 2, 0, st, rows, ldc, key, idx, seg, (int64_t)2, seg);
-  for (int64_t k = 2 * seg; k <= npad; k <<= 1) {
-    for (int64_t j = k >> 1; j >= seg; j >>= 1)
-      mape_detail::launch(bitonic_step_kernel<kFull>, (unsigned)ceil_div(npad, 256), 256, 0, st, rows, ldc, key, idx,
-                          npad, j, k);
-    mape_detail::launch(bitonic_local_kernel<kFull>, nseg, kSeg / 2, 0, st, rows, ldc, key, idx, seg, k, k);
-  }
-}
-
-int sort_row_indices(const int8_t* rows, int ldc, uint32_t* idx, uint64_t* key, int2* runs, unsigned int* counters,
-                     int64_t K, int64_t npad, cudaStream_t st) {
-  if (npad > K) mape_detail::launch(pad_idx_kernel, (unsigned)ceil_div(npad - K, 256), 256, 0, st, idx, K, npad);
-  if (npad < 2) return MAPE_OK;
-  mape_detail::launch(key_rows_kernel, (unsigned)ceil_div(npad, 256), 256, 0, st, rows, ldc, idx, npad, key);
-  bitonic_sort<false>(rows, ldc, idx, key, npad, st);
-  const int64_t runs_cap = K / 2 + 1;
-  MAPE_CUDA_TRY(cudaMemsetAsync(counters, 0, 3 * sizeof(unsigned int), st));
-  mape_detail::launch(key_runs_kernel, (unsigned)ceil_div(K, 256), 256, 0, st, key, K, ldc, runs, runs_cap, counters,
-                      counters + 1, counters + 2);
-  MAPE_LAUNCH_CHECK();
-  unsigned int hc[3] = {0, 0, 0};  // short runs, long runs, longest
-  MAPE_CUDA_TRY(cudaMemcpyAsync(hc, counters, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  MAPE_CUDA_TRY(cudaStreamSynchronize(st));
-  if (hc[2] > (unsigned)kRunMax) {
-    bitonic_sort<true>(rows, ldc, idx, key, npad, st);  // the rows decide every comparison
-  } else {
-    if (hc[0] > 0)
-      mape_detail::launch(run_sort_warp_kernel, (unsigned)ceil_div(hc[0], kRunWarps), 32 * kRunWarps,
-                          (size_t)kRunWarps * kRunWarpBytes, st, rows, ldc, runs, hc[0], idx);
-    if (hc[1] > 0)
-      mape_detail::launch(run_sort_kernel, hc[1], 128, kRunStageBytes, st, rows, ldc, runs + (runs_cap - hc[1]), idx);
-  }
-  MAPE_LAUNCH_CHECK();
-  return MAPE_OK;
+// Sorts the K pairs of the view; the buffer that holds the result.
+int sort_pairs(const SortView& d, cudaStream_t st) {
+  const unsigned tiles = (unsigned)ceil_div(d.K, kSortTile);
+  launch(sort_tiles_kernel, tiles, kSortThreads, 0, st, d);
+  int from = 0;
+  for (int64_t w = kSortTile; w < d.K; w <<= 1, from ^= 1) launch(merge_tiles_kernel, tiles, kSortThreads, 0, st, d, w, from);
+  return from;
 }
 
 uint64_t dedup_table_slots(int64_t count) { return next_pow2((uint64_t)(count > 0 ? count : 1) * 2); }
@@ -437,13 +390,11 @@ extern "C" size_t mape_dedup_workspace_bytes(int64_t count, int32_t ldc) {
   (void)ldc;
   if (count < 0) return 0;
   mape_detail::Sizer s;
-  s.take<uint64_t>((size_t)count);                               // hashes
-  s.take<uint32_t>((size_t)mape_detail::dedup_table_slots(count)); // table
+  s.take<uint64_t>((size_t)count);                               // hashes, then sort keys
+  s.take<uint32_t>((size_t)mape_detail::dedup_table_slots(count)); // table, then sorted indices
   s.take<uint8_t>((size_t)count);                                 // representative flags
-  s.take<uint32_t>((size_t)next_pow2((uint64_t)(count > 0 ? count : 1)));  // sorted indices
-  s.take<uint64_t>((size_t)next_pow2((uint64_t)(count > 0 ? count : 1)));  // their sort keys
-  s.take<int2>((size_t)(count > 0 ? count : 1) / 2 + 1);          // runs of equal keys
-  s.take<unsigned int>(3);                                        // short and long run counts, longest run
+  s.take<uint32_t>((size_t)(count > 0 ? count : 1));              // sorted indices
+  s.take<uint64_t>((size_t)(count > 0 ? count : 1));              // their sort keys
   s.take<unsigned long long>(1);                                  // counter
   return s.bytes();
 }
@@ -462,11 +413,8 @@ extern "C" int mape_dedup(const int8_t* cand, int64_t count, int32_t n, int32_t 
   uint64_t slots = dedup_table_slots(count);
   uint32_t* table = cv.take<uint32_t>((size_t)slots);
   uint8_t* is_rep = cv.take<uint8_t>((size_t)count);
-  uint64_t npad_cap = next_pow2((uint64_t)count);
-  uint32_t* idx = cv.take<uint32_t>((size_t)npad_cap);
-  uint64_t* keys = cv.take<uint64_t>((size_t)npad_cap);
-  int2* runs = cv.take<int2>((size_t)count / 2 + 1);
-  unsigned int* run_counters = cv.take<unsigned int>(3);
+  uint32_t* idx = cv.take<uint32_t>((size_t)count);
+  uint64_t* keys = cv.take<uint64_t>((size_t)count);
   unsigned long long* dK = cv.take<unsigned long long>(1);
   if (!cv.ok) return MAPE_ERR_CAPACITY;
   cudaStream_t st = as_stream(stream);
@@ -483,10 +431,11 @@ extern "C" int mape_dedup(const int8_t* cand, int64_t count, int32_t n, int32_t 
   *K_out = (int64_t)K;
   if ((int64_t)K > uniq_cap) return MAPE_ERR_CAPACITY;
   if (!uniq) return MAPE_ERR_INVALID_ARG;
-  int rc = sort_row_indices(cand, ldc, idx, keys, runs, run_counters, (int64_t)K, (int64_t)next_pow2(K), st);
-  if (rc != MAPE_OK) return rc;
+  // the hashes and the table have served: they are the sort's second buffer
+  const SortView sv{cand, (int64_t)K, ldc, {keys, h}, {idx, table}};
+  const int at = sort_pairs(sv, st);
   int64_t chunks = (int64_t)K * (ldc / 16);
-  mape_detail::launch(gather_rows_kernel, (unsigned)ceil_div(chunks, 256), 256, 0, st, cand, ldc, idx, (int64_t)K, uniq);
+  mape_detail::launch(gather_rows_kernel, (unsigned)ceil_div(chunks, 256), 256, 0, st, cand, ldc, sv.idx[at], (int64_t)K, uniq);
   MAPE_LAUNCH_CHECK();
   MAPE_CUDA_TRY(cudaStreamSynchronize(st));
   return MAPE_OK;
@@ -578,9 +527,8 @@ extern "C" int mape_dedup_static(const int8_t* cand, int64_t count, int32_t n, i
 // output pieces) of all sets, each thread, warp or block finding its set by
 // binary search over the launch's prefix table.  Each set keeps its own hash
 // table, sort arrays and output, carved from its own workspace exactly as
-// mape_dedup carves it, so its output is the same.  The bitonic stages run
-// for the largest set; a set whose sort is already complete at a stage sits
-// it out.
+// mape_dedup carves it, so its output is the same.  The merge passes run for
+// the largest set; a set already sorted is copied along.
 
 namespace {
 
@@ -594,12 +542,13 @@ struct DedupView {
   uint8_t* is_rep;
   uint32_t* idx;
   uint64_t* key;
-  int2* runs;
-  int64_t runs_cap;
   int8_t* uniq;
-  int64_t K, npad, seg;  // distinct rows, sort size, segment of the local stages (0: no sort)
-  int64_t nshort, nlong;  // runs of equal keys for the warp and block sorts
+  int64_t K;  // distinct rows
 };
+
+__device__ __forceinline__ SortView sort_view(const DedupView& d) {
+  return SortView{d.rows, d.K, d.ldc, {d.key, d.h}, {d.idx, d.table}};
+}
 
 __device__ __forceinline__ int find_set(const int64_t* __restrict__ prefix, int count, int64_t x) {
   int lo = 0, hi = count - 1;
@@ -623,71 +572,22 @@ __global__ void hash_insert_batch_kernel(const DedupView* __restrict__ v, const 
   else compact_row(d.is_rep, r, d.idx, K + i);
 }
 
-// prefix: sort positions (npad); the padding sentinel and the keys
-__global__ void key_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix, int count) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= prefix[count]) return;
-  const int i = find_set(prefix, count, t);
-  const DedupView& d = v[i];
-  const int64_t p = t - prefix[i];
-  if (p >= d.K) d.idx[p] = kEmpty;
-  const uint32_t a = d.idx[p];
-  d.key[p] = a == kEmpty ? ~0ull : row_key(d.rows + (int64_t)a * d.ldc);
-}
-
-// prefix: segments (npad / seg); k = 0: the first stages (2 .. seg), else
-// stage k alone (sets with fewer than k positions sit it out)
-__global__ void bitonic_local_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix,
-                                           int count, int64_t k) {
+// prefix: sort tiles
+__global__ void __launch_bounds__(kSortThreads) sort_batch_kernel(const DedupView* __restrict__ v,
+                                                                 const int64_t* __restrict__ prefix, int count) {
   const int i = find_set(prefix, count, blockIdx.x);
-  const DedupView& d = v[i];
-  if (k > d.npad) return;
-  const int64_t kf = k == 0 ? 2 : k, kl = k == 0 ? d.seg : k;
-  bitonic_local_seg<false>(d.rows, d.ldc, d.key, d.idx, d.seg, kf, kl, blockIdx.x - prefix[i]);
+  sort_tile(sort_view(v[i]), blockIdx.x - prefix[i]);
 }
-
-// prefix: sort positions; distance j of stage k
-__global__ void bitonic_step_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix,
-                                          int count, int64_t j, int64_t k) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= prefix[count]) return;
-  const int i = find_set(prefix, count, t);
-  const DedupView& d = v[i];
-  if (k > d.npad) return;
-  bitonic_step_one<false>(d.rows, d.ldc, d.key, d.idx, t - prefix[i], j, k);
-}
-
-// prefix: distinct rows; counters: 3 per set
-__global__ void key_runs_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix, int count,
-                                      unsigned int* __restrict__ counters) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= prefix[count]) return;
-  const int i = find_set(prefix, count, t);
-  const DedupView& d = v[i];
-  unsigned int* c = counters + 3 * i;
-  key_run_at(d.key, d.K, d.ldc, d.runs, d.runs_cap, c, c + 1, c + 2, t - prefix[i]);
-}
-
-// prefix: short runs; one warp per run
-__global__ void run_sort_warp_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix,
-                                           int count) {
-  const int64_t g = (int64_t)blockIdx.x * kRunWarps + (threadIdx.x >> 5);
-  if (g >= prefix[count]) return;  // warp-uniform
-  const int i = find_set(prefix, count, g);
-  const DedupView& d = v[i];
-  run_sort_warp(d.rows, d.ldc, d.runs[g - prefix[i]], d.idx);
-}
-
-// prefix: long runs; one block per run
-__global__ void run_sort_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix, int count) {
+__global__ void __launch_bounds__(kSortThreads) merge_batch_kernel(const DedupView* __restrict__ v,
+                                                                  const int64_t* __restrict__ prefix, int count,
+                                                                  int64_t w, int from) {
   const int i = find_set(prefix, count, blockIdx.x);
-  const DedupView& d = v[i];
-  const int64_t b = blockIdx.x - prefix[i];
-  run_sort_block(d.rows, d.ldc, d.runs[d.runs_cap - d.nlong + b], d.idx);
+  merge_tile(sort_view(v[i]), w, from, blockIdx.x - prefix[i]);
 }
 
 // prefix: 16-byte pieces of the distinct rows
-__global__ void gather_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix, int count) {
+__global__ void gather_batch_kernel(const DedupView* __restrict__ v, const int64_t* __restrict__ prefix, int count,
+                                    int at) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= prefix[count]) return;
   const int i = find_set(prefix, count, t);
@@ -696,13 +596,13 @@ __global__ void gather_batch_kernel(const DedupView* __restrict__ v, const int64
   const int chunks = d.ldc / 16;
   const int64_t r = e / chunks;
   const int c = (int)(e % chunks);
-  reinterpret_cast<uint4*>(d.uniq + r * d.ldc)[c] = reinterpret_cast<const uint4*>(d.rows + (int64_t)d.idx[r] * d.ldc)[c];
+  reinterpret_cast<uint4*>(d.uniq + r * d.ldc)[c] = reinterpret_cast<const uint4*>(d.rows + (int64_t)(at ? d.table : d.idx)[r] * d.ldc)[c];
 }
 
 }  // namespace
 
 // prefix tables of the batch launches, `count` + 1 entries each
-enum { kPxRows, kPxPos, kPxSegs, kPxKeyed, kPxPieces, kPxShort, kPxLong, kPxTables };
+enum { kPxRows, kPxTiles, kPxPieces, kPxTables };
 
 extern "C" size_t mape_dedup_batch_workspace_bytes(int32_t count) {
   if (count <= 0) return 0;
@@ -710,7 +610,6 @@ extern "C" size_t mape_dedup_batch_workspace_bytes(int32_t count) {
   s.take<DedupView>((size_t)count);
   s.take<int64_t>((size_t)kPxTables * (count + 1));  // prefix tables
   s.take<unsigned long long>((size_t)count);         // distinct-row counters
-  s.take<unsigned int>((size_t)3 * count);           // run counters
   return s.bytes();
 }
 
@@ -728,7 +627,6 @@ extern "C" int mape_dedup_batch(mape_dedup_item* items, int32_t count, void* wor
   DedupView* d_views = bc.take<DedupView>((size_t)count);
   int64_t* d_px = bc.take<int64_t>((size_t)kPxTables * (count + 1));
   unsigned long long* d_K = bc.take<unsigned long long>((size_t)count);
-  unsigned int* d_runc = bc.take<unsigned int>((size_t)3 * count);
   if (!bc.ok) return MAPE_ERR_CAPACITY;
   cudaStream_t st = as_stream(stream);
   const int n1 = count + 1;
@@ -760,11 +658,8 @@ extern "C" int mape_dedup_batch(mape_dedup_item* items, int32_t count, void* wor
     d.table = cv.take<uint32_t>((size_t)slots);
     d.mask = slots - 1;
     d.is_rep = cv.take<uint8_t>((size_t)it.count);
-    const uint64_t npad_cap = next_pow2((uint64_t)it.count);
-    d.idx = cv.take<uint32_t>((size_t)npad_cap);
-    d.key = cv.take<uint64_t>((size_t)npad_cap);
-    d.runs = cv.take<int2>((size_t)it.count / 2 + 1);
-    cv.take<unsigned int>(3);
+    d.idx = cv.take<uint32_t>((size_t)it.count);
+    d.key = cv.take<uint64_t>((size_t)it.count);
     cv.take<unsigned long long>(1);
     if (!cv.ok) {
       it.status = MAPE_ERR_CAPACITY;
@@ -787,7 +682,7 @@ extern "C" int mape_dedup_batch(mape_dedup_item* items, int32_t count, void* wor
   MAPE_CUDA_TRY(cudaMemcpyAsync(hK.data(), d_K, sizeof(unsigned long long) * count, cudaMemcpyDeviceToHost, st));
   MAPE_CUDA_TRY(cudaStreamSynchronize(st));
   int first_err = MAPE_OK;
-  int64_t max_npad = 0;
+  int64_t max_K = 0;
   for (int i = 0; i < count; ++i) {
     mape_dedup_item& it = items[i];
     DedupView& d = v[(size_t)i];
@@ -798,67 +693,25 @@ extern "C" int mape_dedup_batch(mape_dedup_item* items, int32_t count, void* wor
       if (first_err == MAPE_OK) first_err = it.status;
       d.K = 0;
     }
-    d.npad = d.K > 0 ? (int64_t)next_pow2((uint64_t)d.K) : 0;
-    d.seg = d.npad >= 2 ? (d.npad < kSeg ? d.npad : kSeg) : 0;
-    d.runs_cap = d.K / 2 + 1;
-    if (d.seg) max_npad = std::max(max_npad, d.npad);
+    max_K = std::max(max_K, d.K);
   }
-  // 2. keys and the bitonic network on them, for the largest set
-  const int64_t pos = prefix(kPxPos, [&](int i) { return v[(size_t)i].npad; });
-  const int64_t segs = prefix(kPxSegs, [&](int i) { return v[(size_t)i].seg ? v[(size_t)i].npad / v[(size_t)i].seg : 0; });
-  const int64_t keyed = prefix(kPxKeyed, [&](int i) { return v[(size_t)i].seg ? v[(size_t)i].K : 0; });
+  // 2. the sort, with the merge passes of the largest set
+  const int64_t tiles = prefix(kPxTiles, [&](int i) { return ceil_div(v[(size_t)i].K, kSortTile); });
   const int64_t pieces = prefix(kPxPieces, [&](int i) { return v[(size_t)i].K * (v[(size_t)i].ldc / 16); });
   MAPE_CUDA_TRY(cudaMemcpyAsync(d_views, v.data(), sizeof(DedupView) * count, cudaMemcpyHostToDevice, st));
-  MAPE_CUDA_TRY(cudaMemcpyAsync(d_px, px.data(), sizeof(int64_t) * kPxShort * n1, cudaMemcpyHostToDevice, st));
-  if (pos > 0)
-    launch(key_batch_kernel, (unsigned)ceil_div(pos, 256), 256, 0, st, (const DedupView*)d_views, dpx(kPxPos),
-           (int)count);
-  if (max_npad >= 2) {
-    launch(bitonic_local_batch_kernel, (unsigned)segs, kSeg / 2, 0, st, (const DedupView*)d_views, dpx(kPxSegs),
-           (int)count, (int64_t)0);
-    for (int64_t k = 2 * kSeg; k <= max_npad; k <<= 1) {
-      for (int64_t j = k >> 1; j >= kSeg; j >>= 1)
-        launch(bitonic_step_batch_kernel, (unsigned)ceil_div(pos, 256), 256, 0, st, (const DedupView*)d_views,
-               dpx(kPxPos), (int)count, j, k);
-      launch(bitonic_local_batch_kernel, (unsigned)segs, kSeg / 2, 0, st, (const DedupView*)d_views, dpx(kPxSegs),
-             (int)count, k);
-    }
-    MAPE_LAUNCH_CHECK();
-    // 3. runs of equal keys, sorted by the rows' remaining bytes
-    MAPE_CUDA_TRY(cudaMemsetAsync(d_runc, 0, sizeof(unsigned int) * 3 * count, st));
-    launch(key_runs_batch_kernel, (unsigned)ceil_div(keyed, 256), 256, 0, st, (const DedupView*)d_views,
-           dpx(kPxKeyed), (int)count, d_runc);
-    MAPE_LAUNCH_CHECK();
-    std::vector<unsigned int> hc((size_t)3 * count, 0);
-    MAPE_CUDA_TRY(cudaMemcpyAsync(hc.data(), d_runc, sizeof(unsigned int) * 3 * count, cudaMemcpyDeviceToHost, st));
-    MAPE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int i = 0; i < count; ++i) {
-      DedupView& d = v[(size_t)i];
-      if (!d.seg) continue;
-      if (hc[(size_t)3 * i + 2] > (unsigned)kRunMax) {  // a run too long for one block: the rows decide every comparison
-        bitonic_sort<true>(d.rows, d.ldc, d.idx, d.key, d.npad, st);
-      } else {
-        d.nshort = hc[(size_t)3 * i];
-        d.nlong = hc[(size_t)3 * i + 1];
-      }
-    }
-    const int64_t nshort = prefix(kPxShort, [&](int i) { return v[(size_t)i].nshort; });
-    const int64_t nlong = prefix(kPxLong, [&](int i) { return v[(size_t)i].nlong; });
-    MAPE_CUDA_TRY(cudaMemcpyAsync(d_views, v.data(), sizeof(DedupView) * count, cudaMemcpyHostToDevice, st));
-    MAPE_CUDA_TRY(cudaMemcpyAsync(d_px + (size_t)kPxShort * n1, px.data() + (size_t)kPxShort * n1,
-                                  sizeof(int64_t) * 2 * n1, cudaMemcpyHostToDevice, st));
-    if (nshort > 0)
-      launch(run_sort_warp_batch_kernel, (unsigned)ceil_div(nshort, kRunWarps), 32 * kRunWarps,
-             (size_t)kRunWarps * kRunWarpBytes, st, (const DedupView*)d_views, dpx(kPxShort), (int)count);
-    if (nlong > 0)
-      launch(run_sort_batch_kernel, (unsigned)nlong, 128, kRunStageBytes, st, (const DedupView*)d_views, dpx(kPxLong),
-             (int)count);
+  MAPE_CUDA_TRY(cudaMemcpyAsync(d_px, px.data(), sizeof(int64_t) * kPxTables * n1, cudaMemcpyHostToDevice, st));
+  int at = 0;
+  if (tiles > 0) {
+    launch(sort_batch_kernel, (unsigned)tiles, kSortThreads, 0, st, (const DedupView*)d_views, dpx(kPxTiles), (int)count);
+    for (int64_t w = kSortTile; w < max_K; w <<= 1, at ^= 1)
+      launch(merge_batch_kernel, (unsigned)tiles, kSortThreads, 0, st, (const DedupView*)d_views, dpx(kPxTiles),
+             (int)count, w, at);
     MAPE_LAUNCH_CHECK();
   }
-  // 4. the distinct rows in order
+  // 3. the distinct rows in order
   if (pieces > 0)
     launch(gather_batch_kernel, (unsigned)ceil_div(pieces, 256), 256, 0, st, (const DedupView*)d_views,
-           dpx(kPxPieces), (int)count);
+           dpx(kPxPieces), (int)count, at);
   MAPE_LAUNCH_CHECK();
   MAPE_CUDA_TRY(cudaStreamSynchronize(st));
   return first_err;
