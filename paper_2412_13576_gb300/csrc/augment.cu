@@ -18,11 +18,19 @@
 //
 // The scoring pass reads every direction once per iteration.  L lanes share a
 // direction (L = 1 .. 32, a power of two): lane j takes the row's 16-byte
-// pieces j, j + L, ..., and the group combines its partial sums (exact int64)
-// and lambda bounds by shuffles; L is autotuned per shape (a few timed score
-// passes on the call's own data, which the pass does not modify) unless the
-// caller fixes it.  A block visits directions in a grid-stride loop, so that
-// at most kMaxScoreBlocks partial minima per start go to the apply pass.
+// pieces j, j + L, ...; L is autotuned per shape (a few timed score passes on
+// the call's own data, which the pass does not modify) unless the caller fixes
+// it.  A block visits directions in a grid-stride loop, so that at most
+// kMaxScoreBlocks partial minima per start go to the apply pass.
+//
+// A direction whose unit step leaves the box both ways (lambda_max < 1 for +g
+// and -g) has no move, and most have none.  So the pass first asks only that,
+// four entries at a time in the bytes of a word (room_fits: about 5 operations
+// an entry against 25 for the sums and bounds), leaving a row at the first
+// piece that rules it out; the directions that remain are queued in shared
+// memory, and full blocks of them get their partial sums (exact int64) and
+// lambda bounds, combined by shuffles.  45 000 directions of n = 200, 64 starts:
+// 0.48 ms an iteration before, 0.16 now.
 //
 // Many instances at once (mape_augment_run_batch): one score and one apply
 // launch per iteration cover the starts of every instance, each block finding
@@ -186,6 +194,7 @@ struct AugView {
 
 constexpr int kScoreThreads = 256;
 constexpr int kMaxScoreBlocks = 1024;  // per start
+constexpr int kScoreBlocks = 1216;     // of a launch over all starts: 8 per SM, each staging its start's tables once
 
 // r = 2 Q x + c and f(x) of start s; checks l <= x <= u.
 __device__ __forceinline__ void init_body(const AugView& v, int s) {
@@ -236,8 +245,30 @@ __device__ __forceinline__ long long floor_div(long long a, long long b) {  // b
 struct ScoreSmem {
   longlong2* rw;
   int2* ud;
+  const uint4* room;    // two per word of 4 coordinates (room_fits; with the pre-pass only)
+  int64_t* queue;       // 2 kScoreThreads directions (with the pre-pass only)
   const uint32_t* rcp;  // rcp[b] = ceil(2^20 / b), b = 1 .. 128
 };
+
+// The unit-step test of 4 entries at once.  With a' = g + 128 in [0, 255], g <= b
+// holds for b >= 0 iff (b + 128) - a' does not borrow, g >= -b iff a' - (128 - b)
+// does not; even and odd bytes go to 16-bit lanes whose bit 8, set in the
+// minuend, survives exactly then.  room[2 w] = up even, up odd, down even, down
+// odd as minuends, room[2 w + 1] = the same as subtrahends 128 - b (rooms above
+// the range of int8 rule nothing out: 127 and 128 stand for them; so do the
+// entries past n).
+constexpr uint32_t kLanes = 0x00FF00FFu, kBit8 = 0x01000100u;
+__device__ __forceinline__ void room_fits(uint32_t g4, const uint4 hi, const uint4 lo, uint32_t& plus, uint32_t& minus) {
+  const uint32_t a = g4 ^ 0x80808080u;
+  const uint32_t e = a & kLanes, o = (a >> 8) & kLanes, eb = e | kBit8, ob = o | kBit8;
+  plus &= (hi.x - e) & (hi.y - o) & (eb - lo.z) & (ob - lo.w);
+  minus &= (hi.z - e) & (hi.w - o) & (eb - lo.x) & (ob - lo.y);
+}
+
+__host__ __device__ inline int score_words(int n) { return (n + 15) / 16 * 4; }
+
+// the pre-pass: where its tables fit beside the others in shared memory
+__host__ __device__ inline bool score_pre(int n) { return n <= 4096; }
 
 // floor(a / b) for 0 <= a < 2048 and 1 <= b <= 128 as (a ceil(2^20 / b)) >> 20:
 // with ceil(2^20 / b) = (2^20 + e) / b, 0 <= e < b, the product is
@@ -256,7 +287,11 @@ __device__ __forceinline__ ScoreSmem stage_start(const AugView& v, int s) {
   const int n = v.n;
   ScoreSmem t;
   t.rw = reinterpret_cast<longlong2*>(smem);                 // 32 n bytes
-  t.ud = reinterpret_cast<int2*>(smem + 4 * (int64_t)n);    // 8 n bytes
+  const int nw = score_words(n);
+  t.ud = reinterpret_cast<int2*>(smem + 4 * (int64_t)n);     // 8 n bytes
+  uint4* room = reinterpret_cast<uint4*>(smem + 5 * (int64_t)n + (n & 1));  // 32 bytes per word
+  t.room = room;
+  t.queue = reinterpret_cast<int64_t*>(room + 2 * (int64_t)nw);
   __shared__ uint32_t s_rcp[129];
   for (int b = threadIdx.x; b <= 128; b += blockDim.x)
     s_rcp[b] = b ? ((1u << kRcpShift) + (uint32_t)b - 1u) / (uint32_t)b : 0u;
@@ -268,6 +303,26 @@ __device__ __forceinline__ ScoreSmem stage_start(const AugView& v, int s) {
     t.rw[2 * i] = make_longlong2(v.R[(int64_t)s * n + i], wi * xi * xi * xi);
     t.rw[2 * i + 1] = make_longlong2(wi * xi * xi, wi * xi);
     t.ud[i] = make_int2(v.u[i] - x[i], x[i] - v.l[i]);
+  }
+  for (int w = threadIdx.x; score_pre(n) && w < nw; w += blockDim.x) {
+    uint32_t hi[2][2] = {{0, 0}, {0, 0}}, lo[2][2] = {{0, 0}, {0, 0}};  // [up, down][even, odd]
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int i = 4 * w + b;
+      int room[2] = {0x7fffffff, 0x7fffffff};
+      if (i < n) {
+        room[0] = v.u[i] - x[i];
+        room[1] = x[i] - v.l[i];
+      }
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int sh = 16 * (b >> 1);
+        hi[c][b & 1] |= (uint32_t)(min(room[c], 127) + 128) << sh;
+        lo[c][b & 1] |= (uint32_t)(128 - min(room[c], 128)) << sh;
+      }
+    }
+    room[2 * w] = make_uint4(hi[0][0] | kBit8, hi[0][1] | kBit8, hi[1][0] | kBit8, hi[1][1] | kBit8);
+    room[2 * w + 1] = make_uint4(lo[0][0], lo[0][1], lo[1][0], lo[1][1]);
   }
   return t;
 }
@@ -346,10 +401,10 @@ __device__ __forceinline__ void score_body(const AugView& v, int s, int bx) {
   const int sub = threadIdx.x % kL;
   const int per_block = blockDim.x / kL;  // directions per block and round
   Best best{kNoMove, kNoMove};
-  for (int64_t k0 = (int64_t)bx * per_block; k0 < v.K; k0 += (int64_t)v.nb * per_block) {  // block-uniform
-    const int64_t k = k0 + threadIdx.x / kL;
+  // the sums and bounds of direction k (k < 0: none), by its group of lanes
+  auto score = [&](int64_t k) {
     DirSums d;
-    if (k < v.K) {
+    if (k >= 0) {
       const int8_t* g = v.G + k * v.ldg;
       if (kVec) {
         for (int p = sub; p * 16 < n; p += kL) {
@@ -380,7 +435,71 @@ __device__ __forceinline__ void score_body(const AugView& v, int s, int bx) {
         d.lam_m = min(d.lam_m, __shfl_xor_sync(0xffffffffu, d.lam_m, o));
       }
     }
-    if (k < v.K && sub == 0) best_move(v, k, d, best);
+    if (k >= 0 && sub == 0) best_move(v, k, d, best);
+  };
+  if (!kVec) {
+    for (int64_t k0 = (int64_t)bx * per_block; k0 < v.K; k0 += (int64_t)v.nb * per_block) {  // block-uniform
+      const int64_t k = k0 + threadIdx.x;
+      score(k < v.K ? k : -1);
+    }
+  } else {
+    // with the pre-pass the directions that remain go through the queue (two
+    // blocks of them at most); without it (score_pre) a round's directions are scored as they come
+    const bool pre = score_pre(n);
+    __shared__ int s_queued;
+    if (threadIdx.x == 0) s_queued = 0;
+    __syncthreads();
+    for (int64_t k0 = (int64_t)bx * per_block;; k0 += (int64_t)v.nb * per_block) {  // block-uniform
+      const bool last = k0 >= v.K;
+      int cnt = last ? 0 : per_block;
+      if (pre) {
+        const int64_t k = k0 + threadIdx.x / kL;
+        uint32_t plus = k < v.K ? kBit8 : 0u, minus = plus;
+        if (k < v.K) {
+          const int8_t* g = v.G + k * v.ldg;
+          for (int p = sub; p * 16 < n; p += kL) {
+            const uint4 q = *reinterpret_cast<const uint4*>(g + p * 16);
+            const uint4* room = t.room + 8 * p;
+            room_fits(q.x, room[0], room[1], plus, minus);
+            room_fits(q.y, room[2], room[3], plus, minus);
+            room_fits(q.z, room[4], room[5], plus, minus);
+            room_fits(q.w, room[6], room[7], plus, minus);
+            if ((plus & kBit8) != kBit8 && (minus & kBit8) != kBit8) break;
+          }
+        }
+        if (kL > 1) {
+#pragma unroll
+          for (int o = kL / 2; o > 0; o >>= 1) {
+            plus &= __shfl_xor_sync(0xffffffffu, plus, o);
+            minus &= __shfl_xor_sync(0xffffffffu, minus, o);
+          }
+        }
+        bool full = false;
+        if (sub == 0 && ((plus & kBit8) == kBit8 || (minus & kBit8) == kBit8)) {
+          const int at = atomicAdd(&s_queued, 1);
+          t.queue[at] = k;
+          full = at >= per_block - 1;
+        }
+        if (!__syncthreads_or(full || last)) continue;
+        cnt = s_queued;
+      }
+      for (int q0 = 0; q0 < cnt; q0 += per_block) {  // a group of lanes each
+        const int q = q0 + threadIdx.x / kL;
+        int64_t k = -1;
+        if (pre) {
+          if (q < cnt) k = t.queue[q];
+        } else if (k0 + q < v.K) {
+          k = k0 + q;
+        }
+        score(k);
+      }
+      if (last) break;
+      if (pre) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_queued = 0;
+        __syncthreads();
+      }
+    }
   }
   // block argmin
   __shared__ Best s_best[32];
@@ -552,12 +671,18 @@ bool valid_lanes(int lanes) {
   return false;
 }
 
-int score_blocks(int64_t K, int lanes) {
+int score_blocks(int64_t K, int S, int lanes) {
   const int64_t per_block = kScoreThreads / lanes;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(K, per_block), kMaxScoreBlocks));
+  const int64_t most = std::min<int64_t>(kMaxScoreBlocks, std::max<int64_t>(8, kScoreBlocks / std::max(S, 1)));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(K, per_block), most));
 }
 
-size_t score_smem(int n) { return (size_t)n * (4 * sizeof(long long) + 2 * sizeof(int32_t)); }
+size_t score_smem(int n) {
+  const size_t tables = (size_t)n * (4 * sizeof(long long) + 2 * sizeof(int32_t));
+  if (!score_pre(n)) return tables;
+  return tables + (n & 1) * sizeof(long long) + (size_t)score_words(n) * 2 * sizeof(uint4) +
+         2 * kScoreThreads * sizeof(int64_t);
+}
 
 // the shared-memory limit of every variant that may take more than 48 KB
 int allow_score_smem(size_t smem, bool batch) {
@@ -601,7 +726,7 @@ AugTuneKey tune_key(int n, int64_t K, int S, bool quartic) {
 AugView make_view(const mape_augment_args* A, long long* R, uint8_t* active, Best* partial, int32_t* iters,
                   unsigned int* n_active, int32_t* bad, int32_t* nmoves, int lanes) {
   AugView v{};
-  v.G = A->G; v.K = A->K; v.ldg = A->ldg; v.n = A->n; v.S = A->S; v.nb = score_blocks(A->K, lanes);
+  v.G = A->G; v.K = A->K; v.ldg = A->ldg; v.n = A->n; v.S = A->S; v.nb = score_blocks(A->K, A->S, lanes);
   v.a = A->a; v.q4 = A->q4; v.qr = A->q_row; v.qc = A->q_col; v.qv = A->q_val; v.nnz = A->nnz;
   v.moves_cap = A->moves_cap;
   v.c = A->c; v.w = A->w; v.l = A->l; v.u = A->u; v.X = A->X; v.fval = A->fval;
@@ -622,7 +747,7 @@ int tune_lanes(const AugView& base, size_t smem, cudaStream_t st, mape_augment_t
   int nc = 0;
   for (int lanes : kLaneChoices) {
     AugView v = base;
-    v.nb = score_blocks(v.K, lanes);
+    v.nb = score_blocks(v.K, v.S, lanes);
     float ms = 0.f;
     for (int rep = 0; rep < 2; ++rep) {  // the first launch loads the kernel
       MAPE_CUDA_TRY(cudaEventRecord(e0, st));
@@ -858,7 +983,7 @@ extern "C" int mape_augment_run(const mape_augment_args* A, int64_t* iters_out, 
   if ((rc = allow_score_smem(smem, false)) != MAPE_OK) return rc;
   int lanes = 1;
   if ((rc = pick_lanes(A, v, vec, smem, st, &lanes)) != MAPE_OK) return rc;
-  v.nb = score_blocks(K, lanes);
+  v.nb = score_blocks(K, S, lanes);
   const ScoreFn score = score_fn(lanes, vec);
   int64_t done_iters = 0;
   const int64_t chunk = 8;
@@ -991,7 +1116,7 @@ extern "C" int mape_augment_run_batch(const mape_augment_args* items, int32_t co
     if ((rc = pick_lanes(&items[big], vb, true, smem, st, &lanes)) != MAPE_OK) return rc;
   }
   for (int i = 0; i < count; ++i) {
-    views[i].nb = score_blocks(items[i].K, lanes);
+    views[i].nb = score_blocks(items[i].K, items[i].S, lanes);
     const int64_t blocks = (items[i].S > 0 && items[i].K > 0) ? (int64_t)views[i].nb * items[i].S : 0;
     blk_prefix[i + 1] = blk_prefix[i] + blocks;
   }
