@@ -7,9 +7,9 @@
 // positions below the start of its own bin.  Each row carries sign-support
 // bitmasks (pos, neg; 64 coordinates per word): h ⊑ g needs pos(h) ⊆ pos(g)
 // and neg(h) ⊆ neg(g); -h ⊑ g needs pos(h) ⊆ neg(g) and neg(h) ⊆ pos(g).  The
-// first mask word rejects almost every pair; survivors get the remaining words
-// and then the magnitude test |h_i| <= |g_i|.  Kept rows are compacted in
-// their input order.
+// signs on the densest coordinates reject almost every pair; survivors get the
+// whole masks and then the magnitude test |h_i| <= |g_i|.  Kept rows are
+// compacted in their input order.
 #include "common.cuh"
 
 #include <algorithm>
@@ -273,16 +273,14 @@ __global__ void bin_scan_kernel(const uint32_t* __restrict__ hist, int nbins, ui
   bin_scan_block(hist, nbins, start, cursor);
 }
 
-// sorted arrays: row index, first mask words, folded signatures, l1
+// sorted arrays: row index, folded signatures, l1
 __device__ __forceinline__ void scatter_row(const int32_t* __restrict__ l1, const uint64_t* __restrict__ masks,
                                             int64_t k, int W, uint32_t* __restrict__ cursor,
-                                            uint32_t* __restrict__ s_idx, uint64_t* __restrict__ s_pk,
-                                            ulonglong2* __restrict__ s_sig, int32_t* __restrict__ s_l1) {
+                                            uint32_t* __restrict__ s_idx, ulonglong2* __restrict__ s_sig,
+                                            int32_t* __restrict__ s_l1) {
   if (l1[k] == kInvalidL1) return;
   uint32_t q = atomicAdd(&cursor[l1[k]], 1u);
   s_idx[q] = (uint32_t)k;
-  // sign masks of coordinates 0..31: pos in the low half, neg in the high half
-  s_pk[q] = (masks[k * 2 * W] & 0xffffffffull) | (masks[k * 2 * W + W] << 32);
   // second filter: every coordinate i folded onto bit i mod 64 (OR of the
   // mask words), pos and neg apart; support and signs of h within those of
   // +-g imply the same for these signatures
@@ -297,11 +295,10 @@ __device__ __forceinline__ void scatter_row(const int32_t* __restrict__ l1, cons
 
 __global__ void scatter_kernel(const int32_t* __restrict__ l1, const uint64_t* __restrict__ masks, int64_t K, int W,
                                uint32_t* __restrict__ cursor, uint32_t* __restrict__ s_idx,
-                               uint64_t* __restrict__ s_pk, ulonglong2* __restrict__ s_sig,
-                               int32_t* __restrict__ s_l1) {
+                               ulonglong2* __restrict__ s_sig, int32_t* __restrict__ s_l1) {
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= K) return;
-  scatter_row(l1, masks, k, W, cursor, s_idx, s_pk, s_sig, s_l1);
+  scatter_row(l1, masks, k, W, cursor, s_idx, s_sig, s_l1);
 }
 
 // ---- sign patterns -------------------------------------------------------------
@@ -317,93 +314,125 @@ __global__ void scatter_kernel(const int32_t* __restrict__ l1, const uint64_t* _
 // order, and every row is compared only with the shorter rows of those
 // lists.  Only pairs that cannot dominate are skipped, so the kept set is the
 // one all pairs give.
+//
+// Within the lists every pair is first tested on the signs of the next 32
+// densest coordinates.  On rows of kernel elements the dense coordinates are
+// those of -C z, which nearly every other row contradicts: of 5450 pairs a row
+// (90 000 rows of 200 entries) 45 pass, where 1780 passed a test on the first
+// 32 coordinates; with 2000 entries none, where 22% did and went on, one lane at a
+// time, to the whole masks.
 
 constexpr int kKeyCoords = 6;
+constexpr int kSieveCoords = 32;  // the next densest, one word of signs each way
+constexpr int kDense = kKeyCoords + kSieveCoords;
 constexpr int kLists = 729;       // 3^kKeyCoords pattern lists
 constexpr int kPartBlock = 1024;  // positions per block of the stable partition
 constexpr int64_t kDensitySample = 16384;  // rows that choose the key coordinates
 
 // per-coordinate nonzero counts of the valid rows among the first rows (64
-// rows per block); any choice of key coordinates gives the same kept set, so
-// a sample is enough to find the densest
-__device__ __forceinline__ void coord_count_block(const int8_t* __restrict__ G, int64_t K, int n, int ldg,
+// rows per block, from their masks); any choice of coordinates gives the same
+// kept set, so a sample is enough to find the densest.  cnt: n counts
+__device__ __forceinline__ void coord_count_block(const uint64_t* __restrict__ masks, int64_t K, int n, int W,
                                                   const int32_t* __restrict__ l1, uint32_t* __restrict__ cnt,
                                                   int64_t bx) {
-  extern __shared__ uint32_t s_cnt[];  // n
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s_cnt[i] = 0;
-  __syncthreads();
+  __shared__ uint8_t s_ok[64];
   const int64_t r0 = bx * 64;
-  for (int64_t e = threadIdx.x; e < 64 * (int64_t)n; e += blockDim.x) {
-    const int64_t k = r0 + e / n;
-    const int i = (int)(e % n);
-    if (k < K && l1[k] != kInvalidL1 && G[k * ldg + i] != 0) atomicAdd(&s_cnt[i], 1u);
+  if (threadIdx.x < 64) s_ok[threadIdx.x] = r0 + threadIdx.x < K && l1[r0 + threadIdx.x] != kInvalidL1;
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const uint64_t* m = masks + r0 * 2 * W + (i >> 6);
+    uint32_t c = 0;
+#pragma unroll 8
+    for (int r = 0; r < 64; ++r)
+      if (s_ok[r]) c += (uint32_t)((m[(int64_t)r * 2 * W] | m[(int64_t)r * 2 * W + W]) >> (i & 63)) & 1u;
+    if (c) atomicAdd(&cnt[i], c);
+  }
+}
+
+__global__ void coord_count_kernel(const uint64_t* __restrict__ masks, int64_t K, int n, int W,
+                                   const int32_t* __restrict__ l1, uint32_t* __restrict__ cnt) {
+  coord_count_block(masks, K, n, W, l1, cnt, blockIdx.x);
+}
+
+// the min(kDense, n) densest coordinates, densest first (ties to the lower
+// index); one block of 1024.  The smallest count that still belongs and, among
+// equals, the last index are found by bisection; those members are then ranked
+// against one another.
+__device__ __forceinline__ void select_keys_block(const uint32_t* __restrict__ cnt, int n,
+                                                  int32_t* __restrict__ keys) {
+  __shared__ uint32_t s_cnt[kDense];
+  __shared__ int s_at[kDense], s_members;
+  const int need = n < kDense ? n : kDense;
+  auto count = [&](auto pred) {
+    int c = 0;
+    for (int b = 0; b < n; b += blockDim.x) {
+      const int i = b + (int)threadIdx.x;
+      c += __syncthreads_count(i < n && pred(cnt[i], i));
+    }
+    return c;
+  };
+  uint32_t t = 0, t_hi = (uint32_t)kDensitySample + 1;  // at least `need` counts >= t, fewer >= t_hi
+  while (t_hi - t > 1) {
+    const uint32_t mid = t + (t_hi - t) / 2;
+    if (count([&](uint32_t c, int) { return c >= mid; }) >= need) t = mid; else t_hi = mid;
+  }
+  int j_lo = -1, j = n - 1;  // members: count > t, or = t and index <= j
+  while (j - j_lo > 1) {
+    const int mid = j_lo + (j - j_lo) / 2;
+    if (count([&](uint32_t c, int i) { return c > t || (c == t && i <= mid); }) >= need) j = mid; else j_lo = mid;
+  }
+  if (threadIdx.x == 0) s_members = 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const uint32_t c = cnt[i];
+    if (c > t || (c == t && i <= j)) {
+      const int q = atomicAdd(&s_members, 1);
+      s_cnt[q] = c;
+      s_at[q] = i;
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x)
-    if (s_cnt[i]) atomicAdd(&cnt[i], s_cnt[i]);
-}
-
-__global__ void coord_count_kernel(const int8_t* __restrict__ G, int64_t K, int n, int ldg,
-                                   const int32_t* __restrict__ l1, uint32_t* __restrict__ cnt) {
-  coord_count_block(G, K, n, ldg, l1, cnt, blockIdx.x);
-}
-
-// the kb densest coordinates (ties to the lower index); one block of 1024
-__device__ __forceinline__ void select_keys_block(const uint32_t* __restrict__ cnt, int n, int kb,
-                                                  int32_t* __restrict__ keys) {
-  __shared__ unsigned long long s_best[32];
-  __shared__ int s_taken[kKeyCoords];
-  for (int b = 0; b < kb; ++b) {
-    // count in the high word, ~index in the low word: the maximum is the
-    // largest count with the lowest index
-    unsigned long long best = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      bool taken = false;
-      for (int c = 0; c < b; ++c) taken |= s_taken[c] == i;
-      if (taken) continue;
-      const unsigned long long v = ((unsigned long long)cnt[i] << 32) | (0xffffffffu - (uint32_t)i) | (1ull << 63);
-      best = v > best ? v : best;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long w = __shfl_xor_sync(0xffffffffu, best, o);
-      best = w > best ? w : best;
-    }
-    if ((threadIdx.x & 31) == 0) s_best[threadIdx.x >> 5] = best;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned long long m = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = s_best[w] > m ? s_best[w] : m;
-      const int idx = (int)(0xffffffffu - (uint32_t)(m & 0xffffffffull));
-      s_taken[b] = idx;
-      keys[b] = idx;
-    }
-    __syncthreads();
+  if ((int)threadIdx.x < need) {
+    int rank = 0;
+    const uint32_t c = s_cnt[threadIdx.x];
+    const int i = s_at[threadIdx.x];
+    for (int q = 0; q < need; ++q) rank += s_cnt[q] > c || (s_cnt[q] == c && s_at[q] < i);
+    keys[rank] = i;
   }
 }
 
-__global__ void select_keys_kernel(const uint32_t* __restrict__ cnt, int n, int kb, int32_t* __restrict__ keys) {
-  select_keys_block(cnt, n, kb, keys);
+__global__ void select_keys_kernel(const uint32_t* __restrict__ cnt, int n, int32_t* __restrict__ keys) {
+  select_keys_block(cnt, n, keys);
 }
 
-// pattern list of the row at sorted position q
-__device__ __forceinline__ void key_row(const int8_t* __restrict__ G, int ldg, const uint32_t* __restrict__ s_idx,
+// pattern list and sieve signs (pos in the low half, neg in the high half) of
+// the row at sorted position q, by a warp
+__device__ __forceinline__ void key_row(const int8_t* __restrict__ G, int n, int ldg, const uint32_t* __restrict__ s_idx,
                                         int64_t q, const int32_t* __restrict__ keys, int kb,
-                                        uint16_t* __restrict__ s_list) {
+                                        uint16_t* __restrict__ s_list, uint64_t* __restrict__ s_pk) {
   const int8_t* g = G + (int64_t)s_idx[q] * ldg;
-  int idx = 0, p3 = 1;
-  for (int b = 0; b < kb; ++b) {
-    const int v = g[keys[b]];
-    idx += (v > 0 ? 1 : (v < 0 ? 2 : 0)) * p3;
-    p3 *= 3;
+  const int lane = threadIdx.x & 31;
+  const int v = kb + lane < n ? g[keys[kb + lane]] : 0;  // kb + lane < kDense
+  const int kv = lane < kb ? g[keys[lane]] : 0;
+  const uint32_t pos = __ballot_sync(0xffffffffu, v > 0), neg = __ballot_sync(0xffffffffu, v < 0);
+  const uint32_t kp = __ballot_sync(0xffffffffu, kv > 0), kn = __ballot_sync(0xffffffffu, kv < 0);
+  if (lane == 0) {
+    int idx = 0, p3 = 1;
+    for (int b = 0; b < kb; ++b) {
+      idx += (int)(((kp >> b) & 1u) + 2u * ((kn >> b) & 1u)) * p3;
+      p3 *= 3;
+    }
+    s_list[q] = (uint16_t)idx;
+    s_pk[q] = (uint64_t)pos | ((uint64_t)neg << 32);
   }
-  s_list[q] = (uint16_t)idx;
 }
 
-__global__ void key_kernel(const int8_t* __restrict__ G, int ldg, const uint32_t* __restrict__ s_idx, int64_t nvalid,
-                           const int32_t* __restrict__ keys, int kb, uint16_t* __restrict__ s_list) {
-  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= nvalid) return;
-  key_row(G, ldg, s_idx, q, keys, kb, s_list);
+__global__ void key_kernel(const int8_t* __restrict__ G, int n, int ldg, const uint32_t* __restrict__ s_idx,
+                           int64_t nvalid, const int32_t* __restrict__ keys, int kb, uint16_t* __restrict__ s_list,
+                           uint64_t* __restrict__ s_pk) {
+  const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (q >= nvalid) return;  // warp-uniform
+  key_row(G, n, ldg, s_idx, q, keys, kb, s_list, s_pk);
 }
 
 // stable partition by list, step 1: counts per (list, block of positions)
@@ -497,15 +526,74 @@ __device__ __forceinline__ bool dominates(const int8_t* __restrict__ G, int n, i
 
 constexpr int kChunk = 4096;  // rows of a source list scanned by one block
 
+// One row g against the source rows [lo, hi) of a list in l1 order: true when
+// one of them dominates it (kSame: h below g, kFlip: -h below g).  The scan is
+// bound by instructions, so rows are taken four at a time from a multiple of
+// four on: one l1 comparison (the largest of the four), two 16-byte loads of
+// sign masks, and one branch for the four mask tests (about 5 instructions a
+// pair; row by row with both orientations' tests it was 11).  225 000 rows of
+// 2000 and 90 000 of 200 entries: 6.16 and 1.27 ms before; 5.74 and 1.2 with
+// this scan, 1.27 and 1.12 with the sieve on dense coordinates too.
+template <bool kSame, bool kFlip>
+__device__ __forceinline__ bool scan_list(const int8_t* __restrict__ G, int n, int ldg, int W,
+                                          const uint64_t* __restrict__ masks, uint32_t lo, uint32_t hi, uint32_t k,
+                                          int32_t gl1, uint32_t np, uint32_t nn, uint64_t gsp, uint64_t gsn,
+                                          const uint32_t* __restrict__ p_idx, const uint64_t* __restrict__ p_pk,
+                                          const ulonglong2* __restrict__ p_sig, const int32_t* __restrict__ p_l1) {
+  // the mask test of one row: 0 in the words that pass
+  auto clash = [&](uint64_t pk, uint32_t& same, uint32_t& flip) {
+    const uint32_t hp = (uint32_t)pk, hn = (uint32_t)(pk >> 32);
+    if (kSame) same = (hp & np) | (hn & nn);
+    if (kFlip) flip = (hp & nn) | (hn & np);
+  };
+  auto full = [&](uint32_t h) {  // signatures, then every coordinate
+    const ulonglong2 hs = p_sig[h];
+    const bool c = (kSame && ((hs.x & gsp) | (hs.y & gsn)) == 0) || (kFlip && ((hs.x & gsn) | (hs.y & gsp)) == 0);
+    return c && dominates(G, n, ldg, W, masks, p_idx[h], k);
+  };
+  auto one = [&](uint32_t h) {
+    uint32_t a = 1, b = 1;
+    clash(p_pk[h], a, b);
+    return ((kSame && a == 0) || (kFlip && b == 0)) && full(h);
+  };
+  uint32_t h = lo;
+  const uint32_t head = min(hi, (lo + 3u) & ~3u);
+  for (; h < head; ++h) {
+    if (p_l1[h] >= gl1) return false;
+    if (one(h)) return true;
+  }
+  for (; h + 4 <= hi && p_l1[h + 3] < gl1; h += 4) {
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(p_pk + h), y = *reinterpret_cast<const ulonglong2*>(p_pk + h + 2);
+    uint32_t a[4] = {1, 1, 1, 1}, b[4] = {1, 1, 1, 1};
+    clash(x.x, a[0], b[0]);
+    clash(x.y, a[1], b[1]);
+    clash(y.x, a[2], b[2]);
+    clash(y.y, a[3], b[3]);
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) any |= (kSame && a[u] == 0) || (kFlip && b[u] == 0);
+    if (any) {
+#pragma unroll 1
+      for (uint32_t u = h; u < h + 4; ++u)
+        if (one(u)) return true;
+    }
+  }
+  for (; h < hi; ++h) {
+    if (p_l1[h] >= gl1) return false;  // the rest of the list is not shorter
+    if (one(h)) return true;
+  }
+  return false;
+}
+
 // Work unit (blockIdx.x, .y, .z): the up to 256 rows of g-block x (a run of
 // one pattern list) against chunk z of one source list.  y = o 2^kb + N: N
 // the key coordinates where the source rows are nonzero (a subset of g's
 // nonzero key coordinates, else the unit is empty), o = 0 for h ⊑ g (g's
 // signs) and o = 1 for -h ⊑ g (reversed signs); N = 0 takes both
 // orientations at once.  Lists are in l1 order, so a row stops at the first
-// source row that is not shorter.  Prefilters per pair: sign masks of
-// coordinates 0..31 packed in one word (pos | neg << 32), then the folded
-// 64-bit signatures of all coordinates, before the full test.  A dominated
+// source row that is not shorter.  Prefilters per pair: the sieve signs packed
+// in one word (pos | neg << 32), then the folded 64-bit signatures of all
+// coordinates, before the full test.  A dominated
 // row gets dom[k] = 1 (several units may write it).
 __device__ __forceinline__ void dominance_block(const int8_t* __restrict__ G, int n, int ldg, int W,
                                                 const uint64_t* __restrict__ masks, const int4 gb,
@@ -547,36 +635,17 @@ __device__ __forceinline__ void dominance_block(const int8_t* __restrict__ G, in
   const uint32_t np = ~(uint32_t)pk, nn = ~(uint32_t)(pk >> 32);
   const ulonglong2 gs = mine ? p_sig[q] : make_ulonglong2(0, 0);
   const uint64_t gsp = ~gs.x, gsn = ~gs.y;
-  const bool want_same = (mode & 1) != 0, want_flip = (mode & 2) != 0;
   if (!mine || dom[k]) return;
   // every thread of the block reads the same source rows at the same time:
-  // the loads are L1 broadcasts, and no block barrier is needed; four rows'
-  // words are loaded at once
-  for (uint32_t h0 = lo; h0 < hi; h0 += 4) {
-    int32_t l1v[4];
-    uint64_t pkv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const bool in = h0 + u < hi;
-      l1v[u] = in ? p_l1[h0 + u] : 0x7fffffff;
-      pkv[u] = in ? p_pk[h0 + u] : 0ull;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (l1v[u] >= gl1) return;  // the rest of the list is not shorter (or past its end)
-      const uint32_t hp = (uint32_t)pkv[u], hn = (uint32_t)(pkv[u] >> 32);
-      const bool cand = (want_same && ((hp & np) | (hn & nn)) == 0) || (want_flip && ((hp & nn) | (hn & np)) == 0);
-      if (!cand) continue;
-      const uint32_t h = h0 + u;
-      const ulonglong2 hs = p_sig[h];
-      const bool cand2 = (want_same && ((hs.x & gsp) | (hs.y & gsn)) == 0) ||
-                         (want_flip && ((hs.x & gsn) | (hs.y & gsp)) == 0);
-      if (cand2 && dominates(G, n, ldg, W, masks, p_idx[h], k)) {
-        dom[k] = 1;
-        return;
-      }
-    }
-  }
+  // the loads are L1 broadcasts, and no block barrier is needed
+  bool d;
+  if (mode == 1)
+    d = scan_list<true, false>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
+  else if (mode == 2)
+    d = scan_list<false, true>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
+  else
+    d = scan_list<true, true>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
+  if (d) dom[k] = 1;
 }
 
 __global__ void dominance_kernel(const int8_t* __restrict__ G, int n, int ldg, int W, const uint64_t* __restrict__ masks,
@@ -921,7 +990,7 @@ extern "C" size_t mape_minimal_workspace_bytes(int64_t K, int32_t n) {
   s.take<ulonglong2>((size_t)K);              //   folded signatures
   s.take<int32_t>((size_t)K);                 //   l1
   s.take<uint32_t>((size_t)n);                // coordinate nonzero counts
-  s.take<int32_t>((size_t)kKeyCoords);        // key coordinates
+  s.take<int32_t>((size_t)kDense);        // key coordinates
   s.take<uint32_t>((size_t)kLists * nblk_part);      // counts per (list, block)
   s.take<uint32_t>((size_t)kLists * nblk_part + 1);  // their exclusive prefix
   s.take<uint32_t>((size_t)kLists + 1);              // list starts
@@ -964,7 +1033,7 @@ extern "C" int mape_minimal_filter(const int8_t* G, int64_t K, int32_t n, int32_
   ulonglong2* p_sig = cv.take<ulonglong2>((size_t)K);
   int32_t* p_l1 = cv.take<int32_t>((size_t)K);
   uint32_t* cnt = cv.take<uint32_t>((size_t)n);
-  int32_t* keys = cv.take<int32_t>((size_t)kKeyCoords);
+  int32_t* keys = cv.take<int32_t>((size_t)kDense);
   uint32_t* bc = cv.take<uint32_t>((size_t)kLists * nblk_part_max);
   uint32_t* boff = cv.take<uint32_t>((size_t)kLists * nblk_part_max + 1);
   uint32_t* lstart = cv.take<uint32_t>((size_t)kLists + 1);
@@ -979,12 +1048,11 @@ extern "C" int mape_minimal_filter(const int8_t* G, int64_t K, int32_t n, int32_
   const unsigned g = (unsigned)ceil_div(K, kTile);
   mape_detail::launch(prep_kernel, g, kTile, 0, st, G, K, n, ldg, W, valid, l1, masks, hist);
   mape_detail::launch(bin_scan_kernel, 1, 1024, 0, st, hist, (int)nb, start, cursor);
-  mape_detail::launch(scatter_kernel, g, kTile, 0, st, l1, masks, K, W, cursor, s_idx, s_pk, s_sig, s_l1);
+  mape_detail::launch(scatter_kernel, g, kTile, 0, st, l1, masks, K, W, cursor, s_idx, s_sig, s_l1);
   mape_detail::launch(clear_keep_kernel, g, kTile, 0, st, keep, K);
   const int64_t K_sample = K < kDensitySample ? K : kDensitySample;
-  mape_detail::launch(coord_count_kernel, (unsigned)ceil_div(K_sample, 64), 256, sizeof(uint32_t) * n, st, G, K_sample,
-                      n, ldg, l1, cnt);
-  mape_detail::launch(select_keys_kernel, 1, 1024, 0, st, cnt, n, kb, keys);
+  mape_detail::launch(coord_count_kernel, (unsigned)ceil_div(K_sample, 64), 256, 0, st, masks, K_sample, n, W, l1, cnt);
+  mape_detail::launch(select_keys_kernel, 1, 1024, 0, st, cnt, n, keys);
   MAPE_LAUNCH_CHECK();
   // number of valid rows = end of the last bin
   uint32_t last_start = 0, last_count = 0;
@@ -995,8 +1063,8 @@ extern "C" int mape_minimal_filter(const int8_t* G, int64_t K, int32_t n, int32_
   if (nvalid > 0) {
     // pattern lists, each in l1 order (stable partition of the l1 order)
     const int nblk_part = (int)ceil_div(nvalid, kPartBlock);
-    mape_detail::launch(key_kernel, (unsigned)ceil_div(nvalid, kTile), kTile, 0, st, G, ldg, s_idx, nvalid, keys, kb,
-                        s_list);
+    mape_detail::launch(key_kernel, (unsigned)ceil_div(nvalid, kTile / 32), kTile, 0, st, G, n, ldg, s_idx, nvalid,
+                        keys, kb, s_list, s_pk);
     mape_detail::launch(part_count_kernel, (unsigned)nblk_part, kPartBlock, 0, st, s_list, nvalid, nlists, nblk_part,
                         bc);
     mape_detail::launch(bin_scan_kernel, 1, 1024, 0, st, bc, nlists * nblk_part, boff, boff);
@@ -1083,7 +1151,7 @@ __global__ void min_rows_batch_kernel(const MinView* __restrict__ v, const int64
   const MinView& d = v[i];
   const int64_t k = t - prefix[i];
   if (phase == 0) prep_row(d.G, k, d.n, d.ldg, d.W, d.valid, d.l1, d.masks, d.hist);
-  else if (phase == 1) scatter_row(d.l1, d.masks, k, d.W, d.cursor, d.s_idx, d.s_pk, d.s_sig, d.s_l1);
+  else if (phase == 1) scatter_row(d.l1, d.masks, k, d.W, d.cursor, d.s_idx, d.s_sig, d.s_l1);
   else if (phase == 2) d.keep[k] = 0;
   else d.keep[k] = (d.l1[k] != kInvalidL1 && !d.keep[k]) ? 1 : 0;
 }
@@ -1107,7 +1175,7 @@ __global__ void min_keys_batch_kernel(const MinView* __restrict__ v, int64_t* __
     if (threadIdx.x == 0) nvalid[blockIdx.x] = 0;
     return;
   }
-  select_keys_block(d.cnt, d.n, d.kb, d.keys);
+  select_keys_block(d.cnt, d.n, d.keys);
   if (threadIdx.x == 0) nvalid[blockIdx.x] = (int64_t)d.start[d.nb - 1] + d.hist[d.nb - 1];
 }
 
@@ -1115,17 +1183,17 @@ __global__ void min_keys_batch_kernel(const MinView* __restrict__ v, int64_t* __
 __global__ void min_coord_batch_kernel(const MinView* __restrict__ v, const int64_t* __restrict__ prefix, int count) {
   const int i = find_inst(prefix, count, blockIdx.x);
   const MinView& d = v[i];
-  coord_count_block(d.G, d.K_sample, d.n, d.ldg, d.l1, d.cnt, blockIdx.x - prefix[i]);
+  coord_count_block(d.masks, d.K_sample, d.n, d.W, d.l1, d.cnt, blockIdx.x - prefix[i]);
 }
 
-// prefix: valid rows (pattern list of each)
+// prefix: valid rows (pattern list and sieve signs of each), a warp per row
 __global__ void min_key_rows_batch_kernel(const MinView* __restrict__ v, const int64_t* __restrict__ prefix,
                                           int count) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= prefix[count]) return;
+  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (t >= prefix[count]) return;  // warp-uniform
   const int i = find_inst(prefix, count, t);
   const MinView& d = v[i];
-  key_row(d.G, d.ldg, d.s_idx, t - prefix[i], d.keys, d.kb, d.s_list);
+  key_row(d.G, d.n, d.ldg, d.s_idx, t - prefix[i], d.keys, d.kb, d.s_list, d.s_pk);
 }
 
 // prefix: partition blocks; phase 0 counts, 1 scatters
@@ -1219,7 +1287,6 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
   };
   auto dpx = [&](int t) -> const int64_t* { return d_px + (size_t)t * n1; };
   std::vector<MinView> v((size_t)count);
-  int max_n = 1;
   for (int i = 0; i < count; ++i) {
     mape_minimal_item& it = items[i];
     it.K_out = 0;
@@ -1237,7 +1304,6 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
     d.nlists = 1;
     for (int b = 0; b < d.kb; ++b) d.nlists *= 3;
     d.K_sample = K < kDensitySample ? K : kDensitySample;
-    max_n = std::max(max_n, n);
     // the same carve as mape_minimal_filter
     Carver cv(it.workspace, it.workspace_bytes);
     d.l1 = cv.take<int32_t>((size_t)K);
@@ -1255,7 +1321,7 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
     d.p_sig = cv.take<ulonglong2>((size_t)K);
     d.p_l1 = cv.take<int32_t>((size_t)K);
     d.cnt = cv.take<uint32_t>((size_t)n);
-    d.keys = cv.take<int32_t>((size_t)kKeyCoords);
+    d.keys = cv.take<int32_t>((size_t)kDense);
     d.bc = cv.take<uint32_t>((size_t)kLists * nblk_part_max);
     d.boff = cv.take<uint32_t>((size_t)kLists * nblk_part_max + 1);
     d.lstart = cv.take<uint32_t>((size_t)kLists + 1);
@@ -1281,7 +1347,7 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
   launch(min_scan_batch_kernel, (unsigned)count, 1024, 0, st, cv_, 0);
   launch(min_rows_batch_kernel, gr, kTile, 0, st, cv_, dpx(kRows), (int)count, 1);
   launch(min_rows_batch_kernel, gr, kTile, 0, st, cv_, dpx(kRows), (int)count, 2);
-  launch(min_coord_batch_kernel, (unsigned)cblocks, 256, sizeof(uint32_t) * max_n, st, cv_, dpx(kCoord), (int)count);
+  launch(min_coord_batch_kernel, (unsigned)cblocks, 256, 0, st, cv_, dpx(kCoord), (int)count);
   launch(min_keys_batch_kernel, (unsigned)count, 1024, 0, st, cv_, d_nvalid);
   MAPE_LAUNCH_CHECK();
   std::vector<int64_t> nvalid((size_t)count, 0);
@@ -1299,7 +1365,7 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
     MAPE_CUDA_TRY(cudaMemcpyAsync(d_views, v.data(), sizeof(MinView) * count, cudaMemcpyHostToDevice, st));
     MAPE_CUDA_TRY(cudaMemcpyAsync(d_px + (size_t)kValid * n1, px.data() + (size_t)kValid * n1,
                                   sizeof(int64_t) * 3 * n1, cudaMemcpyHostToDevice, st));
-    launch(min_key_rows_batch_kernel, (unsigned)ceil_div(valid_rows, kTile), kTile, 0, st, cv_, dpx(kValid),
+    launch(min_key_rows_batch_kernel, (unsigned)ceil_div(valid_rows, kTile / 32), kTile, 0, st, cv_, dpx(kValid),
            (int)count);
     launch(min_part_batch_kernel, (unsigned)pblocks, kPartBlock, 0, st, cv_, dpx(kPart), (int)count, 0);
     launch(min_scan_batch_kernel, (unsigned)count, 1024, 0, st, cv_, 1);
