@@ -11,6 +11,7 @@
 // whole masks and then the magnitude test |h_i| <= |g_i|.  Kept rows are
 // compacted in their input order.
 #include "common.cuh"
+#include "rows_tile.cuh"
 
 #include <algorithm>
 #include <vector>
@@ -79,35 +80,123 @@ __global__ void kernel_test_kernel(const int32_t* __restrict__ A, int m, int n, 
 }
 
 // A in compressed rows (CSR), for the test of rows too long for the dp4a path:
-// row r's nonzeros are col[rowptr[r] .. rowptr[r+1]), val[...] in column order.
-// One warp per row of A.
-__global__ void csr_count_kernel(const int32_t* __restrict__ A, int m, int n, uint32_t* __restrict__ rowcnt) {
+// row r's nonzeros are entries rowptr[r] .. rowptr[r+1] in column order, one
+// warp per row of A.  When every row of A has sum |a| <= kTileSum they are
+// packed for the tile kernel (pack[q] = tile_at(column) | value << kTileShift,
+// start[r] = the sum's start, see there); else *big is set and they are col, val.
+// A row of a small sum (at most 255 entries, fewer than n) is filled up with
+// zero entries to a multiple of four.
+constexpr int kTileSum = 255, kTileShift = 17;
+
+__global__ void csr_count_kernel(const int32_t* __restrict__ A, int m, int n, uint32_t* __restrict__ rowcnt,
+                                 int32_t* __restrict__ big) {
   const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= m) return;
   uint32_t c = 0;
-  for (int i = lane; i < n; i += 32) c += A[(int64_t)r * n + i] != 0;
-  for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-  if (lane == 0) rowcnt[r] = c;
+  unsigned long long sum = 0;
+  for (int i = lane; i < n; i += 32) {
+    const long long v = A[(int64_t)r * n + i];
+    c += v != 0;
+    sum += (unsigned long long)(v < 0 ? -v : v);
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    c += __shfl_xor_sync(0xffffffffu, c, off);
+    sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  }
+  if (lane == 0) {
+    rowcnt[r] = sum > kTileSum ? c : (c + 3) & ~3u;
+    if (sum > kTileSum) atomicOr(big, 1);
+  }
 }
 
+// start: the counts' array, read by the scan before
 __global__ void csr_fill_kernel(const int32_t* __restrict__ A, int m, int n, const uint32_t* __restrict__ rowptr,
-                                uint16_t* __restrict__ col, int32_t* __restrict__ val) {
+                                uint16_t* __restrict__ col, int32_t* __restrict__ val, const int32_t* __restrict__ big,
+                                uint32_t* __restrict__ pack, uint32_t* __restrict__ start) {
   const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= m) return;
-  uint32_t pos = rowptr[r];
+  const bool packed = *big == 0;
+  uint32_t pos = rowptr[r], sum = 0;
   for (int i0 = 0; i0 < n; i0 += 32) {
     const int i = i0 + lane;
     const int v = i < n ? A[(int64_t)r * n + i] : 0;
     const unsigned bal = __ballot_sync(0xffffffffu, v != 0);
     if (v != 0) {
       const uint32_t q = pos + __popc(bal & ((1u << lane) - 1));
-      col[q] = (uint16_t)i;
-      val[q] = v;
+      if (packed) {
+        pack[q] = tile_at(i) | ((uint32_t)v << kTileShift);
+        sum += (uint32_t)v;
+      } else {
+        col[q] = (uint16_t)i;
+        val[q] = v;
+      }
     }
     pos += __popc(bal);
   }
+  const uint32_t q = pos + lane;
+  if (q < rowptr[r + 1]) {  // at most three
+    if (packed) {
+      pack[q] = 0;
+    } else {
+      col[q] = 0;
+      val[q] = 0;
+    }
+  }
+  if (!packed) return;
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  if (lane == 0) start[r] = 0u - 128u * 65537u * sum;
+}
+
+// A g over tiles of 32 candidate rows (rows_tile.cuh, bytes g + 128): eight
+// lanes take a row of A, each with four candidates in two words of 16-bit sums,
+// candidates 0 and 2 of a word in its halves: word += a_rc (g_0 + 2^16 g_2),
+// started at -128 sum a_rc in both halves.  With sum |a_rc| <= 255 every sum lies
+// within +-32640, so the word is S_0 + 2^16 S_2 mod 2^32 for exactly one pair of
+// sums, and zero exactly when both are.  A warp has 32 rows' products per
+// shared-memory word instead of a byte load each, whose bank conflicts bound
+// the warp-per-rows kernel below: 1.54 ms for 225 000 rows against 400 x 2000 (6804
+// nonzeros), 0.31 ms here.
+__global__ void __launch_bounds__(512)
+kernel_test_tile_kernel(const uint32_t* __restrict__ rowptr, const uint32_t* __restrict__ pack,
+                        const uint32_t* __restrict__ start, const int32_t* __restrict__ big, int m, int n,
+                        const int8_t* __restrict__ G, int64_t K, int ldg, uint8_t* __restrict__ ok,
+                        unsigned long long* __restrict__ fails) {
+  if (*big != 0) return;
+  extern __shared__ __align__(16) char s_tile[];
+  __shared__ uint32_t s_bad;
+  const int64_t k0 = (int64_t)blockIdx.x * kTileRows;
+  const int cnt = (int)(K - k0 < kTileRows ? K - k0 : kTileRows);
+  if (threadIdx.x == 0) s_bad = 0;
+  stage_tile<true>(G, k0, cnt, n, ldg, s_tile);
+  __syncthreads();
+  const uint32_t q = threadIdx.x % kTileLanes, turn = q << 4;
+  uint32_t bad = 0;
+  for (int r = threadIdx.x / kTileLanes; r < m; r += blockDim.x / kTileLanes) {
+    uint32_t even = start[r], odd = even;
+    const uint32_t e1 = rowptr[r + 1];
+    for (uint32_t e = rowptr[r]; e < e1; e += 4) {
+      const uint4 a4 = *reinterpret_cast<const uint4*>(pack + e);
+      const uint32_t a[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const uint32_t x = *reinterpret_cast<const uint32_t*>(s_tile + ((a[b] & ((1u << kTileShift) - 1)) ^ turn));
+        const uint32_t v = (uint32_t)((int32_t)a[b] >> kTileShift);
+        even += v * (x & 0x00FF00FFu);
+        odd += v * __byte_perm(x, 0u, 0x4341);
+      }
+    }
+    // the lower sum, and what is left of the upper half without it
+    if ((even | odd) != 0) {
+      const uint32_t el = (uint32_t)(int32_t)(int16_t)even, ol = (uint32_t)(int32_t)(int16_t)odd;
+      bad |= (el ? 1u : 0u) | (ol ? 2u : 0u) | (even != el ? 4u : 0u) | (odd != ol ? 8u : 0u);
+    }
+  }
+  if (bad) atomicOr(&s_bad, bad << (4 * q));
+  __syncthreads();
+  if ((int)threadIdx.x < cnt) ok[k0 + threadIdx.x] = (s_bad >> threadIdx.x) & 1u ? 0 : 1;
+  if (threadIdx.x == 0 && s_bad) atomicAdd(fails, (unsigned long long)__popc(s_bad));
 }
 
 // A g over rows staged in shared memory, one warp per group of candidate
@@ -163,7 +252,9 @@ __device__ __forceinline__ void csr_test_rows(const uint32_t* __restrict__ rowpt
 __global__ void __launch_bounds__(32 * kCsrWarps)
 kernel_test_csr_kernel(const uint32_t* __restrict__ rowptr, const uint16_t* __restrict__ col,
                        const int32_t* __restrict__ val, int m, const int8_t* __restrict__ G, int64_t K,
-                       int ldg, uint8_t* __restrict__ ok, unsigned long long* __restrict__ fails) {
+                       int ldg, const int32_t* __restrict__ big, uint8_t* __restrict__ ok,
+                       unsigned long long* __restrict__ fails) {
+  if (*big == 0) return;  // the tile kernel's
   extern __shared__ __align__(16) int8_t s_rows[];
   const int w = threadIdx.x >> 5;
   int8_t* rows = s_rows + (size_t)w * kCsrRows * ldg;
@@ -775,7 +866,7 @@ int64_t l1_bins(int32_t n) { return (int64_t)127 * n + 1; }
 extern "C" size_t mape_kernel_test_workspace_bytes(int32_t m, int32_t n) {
   if (m <= 0 || n <= 0) return 0;
   mape_detail::Sizer s;
-  s.take<unsigned long long>(1);             // failure counter
+  s.take<unsigned long long>(2);             // failure counter, large-row flag
   s.take<uint32_t>((size_t)m + 1);           // nonzeros per row of A
   s.take<uint32_t>((size_t)m + 1);           // row starts
   s.take<uint16_t>((size_t)m * n);           // column indices
@@ -793,7 +884,7 @@ extern "C" int mape_kernel_test(const int32_t* A, int32_t m, int32_t n, const in
   *fail_count = 0;
   if (K == 0) return MAPE_OK;
   Carver cv(workspace, workspace_bytes);
-  unsigned long long* d_fail = cv.take<unsigned long long>(1);
+  unsigned long long* d_fail = cv.take<unsigned long long>(2);  // and the large-row flag
   uint32_t* rowcnt = cv.take<uint32_t>((size_t)m + 1);
   uint32_t* rowptr = cv.take<uint32_t>((size_t)m + 1);
   uint16_t* col = cv.take<uint16_t>((size_t)m * n);
@@ -801,17 +892,30 @@ extern "C" int mape_kernel_test(const int32_t* A, int32_t m, int32_t n, const in
   if (!cv.ok) return MAPE_ERR_CAPACITY;
   cudaStream_t st = as_stream(stream);
   const int stage8 = ((int64_t)m * ldg <= 48 * 1024 && ldg <= kMaxRegRow) ? 1 : 0;
-  MAPE_CUDA_TRY(cudaMemsetAsync(d_fail, 0, sizeof(unsigned long long), st));
+  MAPE_CUDA_TRY(cudaMemsetAsync(d_fail, 0, 2 * sizeof(unsigned long long), st));
   if (stage8) {
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(K, 128), 152 * 4);
     mape_detail::launch(kernel_test_kernel, grid, 128, (size_t)m * ldg, st, A, m, n, G, K, ldg, stage8, ok, d_fail);
   } else {
     const unsigned gw = (unsigned)ceil_div((int64_t)m * 32, 256);
     MAPE_CUDA_TRY(cudaMemsetAsync(rowcnt, 0, sizeof(uint32_t) * ((size_t)m + 1), st));
-    mape_detail::launch(csr_count_kernel, gw, 256, 0, st, A, m, n, rowcnt);
+    int32_t* big = reinterpret_cast<int32_t*>(d_fail + 1);
+    mape_detail::launch(csr_count_kernel, gw, 256, 0, st, A, m, n, rowcnt, big);
     // exclusive prefix over m + 1 entries: entry m = nnz(A)
     mape_detail::launch(bin_scan_kernel, 1, 1024, 0, st, rowcnt, m + 1, rowptr, rowptr);
-    mape_detail::launch(csr_fill_kernel, gw, 256, 0, st, A, m, n, rowptr, col, val);
+    uint32_t* pack = reinterpret_cast<uint32_t*>(val);
+    mape_detail::launch(csr_fill_kernel, gw, 256, 0, st, A, m, n, rowptr, col, val, big, pack, rowcnt);
+    // the device decides which of the two kernels works, the call does not wait for it
+    const size_t tile = tile_bytes(n);
+    if (tile > 48 * 1024) {
+      size_t lim = 0;
+      const int rc = allow_max_dynamic_smem((const void*)kernel_test_tile_kernel, &lim);
+      if (rc != MAPE_OK) return rc;
+      if (tile > lim) return MAPE_ERR_SHAPE;
+    }
+    // three blocks of 256 an SM up to 75 KB, else one of 512
+    mape_detail::launch(kernel_test_tile_kernel, (unsigned)ceil_div(K, kTileRows), tile > 75 * 1024 ? 512 : 256, tile, st,
+                        rowptr, pack, rowcnt, big, m, n, G, K, ldg, ok, d_fail);
     const size_t smem = (size_t)kCsrWarps * kCsrRows * ldg;
     if (smem > 48 * 1024) {
       size_t lim = 0;
@@ -820,8 +924,8 @@ extern "C" int mape_kernel_test(const int32_t* A, int32_t m, int32_t n, const in
       if (smem > lim) return MAPE_ERR_SHAPE;
     }
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(K, (int64_t)kCsrWarps * kCsrRows), 152 * 4);
-    mape_detail::launch(kernel_test_csr_kernel, grid, 32 * kCsrWarps, smem, st, rowptr, col, val, m, G, K, ldg, ok,
-                        d_fail);
+    mape_detail::launch(kernel_test_csr_kernel, grid, 32 * kCsrWarps, smem, st, rowptr, col, val, m, G, K, ldg, big,
+                        ok, d_fail);
   }
   MAPE_LAUNCH_CHECK();
   unsigned long long f = 0;
