@@ -655,12 +655,13 @@ constexpr int kChunk = 4096;  // rows of a source list scanned by one block
 
 // One row g against the source rows [lo, hi) of a list in l1 order: true when
 // one of them dominates it (kSame: h below g, kFlip: -h below g).  The scan is
-// bound by instructions, so rows are taken four at a time from a multiple of
-// four on: one l1 comparison (the largest of the four), two 16-byte loads of
-// sign masks, and one branch for the four mask tests (about 5 instructions a
+// bound by instructions, so rows are taken eight at a time from an even
+// one on: one l1 comparison (the largest of the eight), four 16-byte loads of
+// sign masks, and one branch for the eight mask tests (about 5 instructions a
 // pair; row by row with both orientations' tests it was 11).  225 000 rows of
-// 2000 and 90 000 of 200 entries: 6.16 and 1.27 ms before; 5.74 and 1.2 with
-// this scan, 1.27 and 1.12 with the sieve on dense coordinates too.
+// 2000 and 90 000 of 200 entries: 6.16 and 1.27 ms before; 1.27 and 1.12 by
+// fours with the sieve on dense coordinates, 1.04 and 0.41 with the magnitudes
+// by 16 bytes and the units below, 0.86 and 0.36 by eights.
 template <bool kSame, bool kFlip>
 __device__ __forceinline__ bool scan_list(const int8_t* __restrict__ G, int n, int ldg, int W,
                                           const uint64_t* __restrict__ masks, uint32_t lo, uint32_t hi, uint32_t k,
@@ -684,24 +685,26 @@ __device__ __forceinline__ bool scan_list(const int8_t* __restrict__ G, int n, i
     return ((kSame && a == 0) || (kFlip && b == 0)) && full(h);
   };
   uint32_t h = lo;
-  const uint32_t head = min(hi, (lo + 3u) & ~3u);
+  const uint32_t head = min(hi, (lo + 1u) & ~1u);
   for (; h < head; ++h) {
     if (p_l1[h] >= gl1) return false;
     if (one(h)) return true;
   }
-  for (; h + 4 <= hi && p_l1[h + 3] < gl1; h += 4) {
-    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(p_pk + h), y = *reinterpret_cast<const ulonglong2*>(p_pk + h + 2);
-    uint32_t a[4] = {1, 1, 1, 1}, b[4] = {1, 1, 1, 1};
-    clash(x.x, a[0], b[0]);
-    clash(x.y, a[1], b[1]);
-    clash(y.x, a[2], b[2]);
-    clash(y.y, a[3], b[3]);
+  for (; h + 8 <= hi && p_l1[h + 7] < gl1; h += 8) {
+    ulonglong2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = *reinterpret_cast<const ulonglong2*>(p_pk + h + 2 * u);
     bool any = false;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) any |= (kSame && a[u] == 0) || (kFlip && b[u] == 0);
+    for (int u = 0; u < 4; ++u) {
+      uint32_t a0 = 1, b0 = 1, a1 = 1, b1 = 1;
+      clash(x[u].x, a0, b0);
+      clash(x[u].y, a1, b1);
+      any |= (kSame && (a0 == 0 || a1 == 0)) || (kFlip && (b0 == 0 || b1 == 0));
+    }
     if (any) {
 #pragma unroll 1
-      for (uint32_t u = h; u < h + 4; ++u)
+      for (uint32_t u = h; u < h + 8; ++u)
         if (one(u)) return true;
     }
   }
@@ -712,74 +715,91 @@ __device__ __forceinline__ bool scan_list(const int8_t* __restrict__ G, int n, i
   return false;
 }
 
-// Work unit (blockIdx.x, .y, .z): the up to 256 rows of g-block x (a run of
-// one pattern list) against chunk z of one source list.  y = o 2^kb + N: N
-// the key coordinates where the source rows are nonzero (a subset of g's
-// nonzero key coordinates, else the unit is empty), o = 0 for h ⊑ g (g's
-// signs) and o = 1 for -h ⊑ g (reversed signs); N = 0 takes both
-// orientations at once.  Lists are in l1 order, so a row stops at the first
-// source row that is not shorter.  Prefilters per pair: the sieve signs packed
-// in one word (pos | neg << 32), then the folded 64-bit signatures of all
-// coordinates, before the full test.  A dominated
-// row gets dom[k] = 1 (several units may write it).
+// Block (x, y, z): the up to 256 rows of g-block x (a run of one pattern
+// list), a thread each, against chunk z of the source lists of its work units
+// y, y + kUnitSplit, ....  Unit 0 is N = 0, N being the key coordinates where the
+// source rows are nonzero, with both orientations at once; then each nonempty
+// subset N of g's nonzero key coordinates has two units, o = 0 for h ⊑ g
+// (g's signs) and o = 1 for -h ⊑ g (reversed signs).  Short source rows, which
+// dominate most, come first.  (A block for each of the 2 x 64 subsets of the six
+// key coordinates, most of them not g's, took half the instructions of 90 000
+// rows of 200 entries: 0.66 ms, 0.36 now with the longer
+// strides of the scan; 1.4 -> 0.86 ms for 225 000 rows of 2000.)  Lists are in l1 order, so a
+// row stops at the first source row that is not shorter.  Prefilters per pair:
+// the sieve signs packed in one word (pos | neg << 32), then the folded 64-bit
+// signatures of all coordinates, before the full test.  A dominated row gets
+// dom[k] = 1 (several units may write it).
+constexpr int kUnitSplit = 8;
+
 __device__ __forceinline__ void dominance_block(const int8_t* __restrict__ G, int n, int ldg, int W,
                                                 const uint64_t* __restrict__ masks, const int4 gb,
                                                 const uint32_t* __restrict__ lstart, int kb,
                                                 const uint32_t* __restrict__ p_idx, const uint64_t* __restrict__ p_pk,
                                                 const ulonglong2* __restrict__ p_sig, const int32_t* __restrict__ p_l1,
-                                                uint8_t* __restrict__ dom, int by, int bz) {
-  __shared__ int s_maxl1;
-  const int nsub = 1 << kb;
-  if (by >= 2 * nsub) return;  // batch: a unit beyond this instance's orientations and subsets
-  const int o = by / nsub, N = by % nsub;
-  // g's pattern digits; the source pattern keeps digits in N (reversed for o = 1)
-  int nzmask = 0, S = 0;
-  {
-    int rest = gb.z, p3 = 1;
-    for (int b = 0; b < kb; ++b) {
-      const int t = rest % 3;
-      rest /= 3;
-      if (t != 0) nzmask |= 1 << b;
-      if ((N >> b) & 1) S += (o == 0 ? t : 3 - t) * p3;
-      p3 *= 3;
-    }
-  }
-  if ((N & ~nzmask) != 0 || (N == 0 && o == 1)) return;  // uniform over the block
-  const int mode = N == 0 ? 3 : (o == 0 ? 1 : 2);  // bit 0: h ⊑ g, bit 1: -h ⊑ g
-  const uint32_t lo = lstart[S] + (uint32_t)bz * (uint32_t)kChunk, s_end = lstart[S + 1];
-  if (lo >= s_end) return;
-  const uint32_t hi = lo + kChunk < s_end ? lo + kChunk : s_end;
+                                                volatile uint8_t* __restrict__ dom, int by, int bz) {
+  if ((int)((threadIdx.x & ~31u)) >= gb.y) return;  // no row for the warp
   const bool mine = (int)threadIdx.x < gb.y;
   const uint32_t q = (uint32_t)gb.x + threadIdx.x;
-  const int32_t gl1 = mine ? p_l1[q] : 0;
-  if (threadIdx.x == 0) s_maxl1 = 0;
-  __syncthreads();
-  if (mine) atomicMax(&s_maxl1, gl1);
-  __syncthreads();
-  if (p_l1[lo] >= s_maxl1) return;  // no source row of the chunk is shorter than any g
   const uint32_t k = mine ? p_idx[q] : 0;
+  const int32_t gl1 = mine ? p_l1[q] : 0;
+  const int32_t longest = __reduce_max_sync(0xffffffffu, gl1);
   const uint64_t pk = mine ? p_pk[q] : 0;
   const uint32_t np = ~(uint32_t)pk, nn = ~(uint32_t)(pk >> 32);
   const ulonglong2 gs = mine ? p_sig[q] : make_ulonglong2(0, 0);
   const uint64_t gsp = ~gs.x, gsn = ~gs.y;
-  if (!mine || dom[k]) return;
-  // every thread of the block reads the same source rows at the same time:
-  // the loads are L1 broadcasts, and no block barrier is needed
-  bool d;
-  if (mode == 1)
-    d = scan_list<true, false>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
-  else if (mode == 2)
-    d = scan_list<false, true>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
-  else
-    d = scan_list<true, true>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
-  if (d) dom[k] = 1;
+  // g's pattern: bits b of the nonzero and of the negative key coordinates
+  uint32_t nzmask = 0, minus = 0;
+  {
+    int rest = gb.z;
+    for (int b = 0; b < kb; ++b) {
+      const int t = rest % 3;
+      rest /= 3;
+      if (t != 0) nzmask |= 1u << b;
+      if (t == 2) minus |= 1u << b;
+    }
+  }
+  const int units = 2 * (1 << __popc(nzmask)) - 1;
+  for (int u = by; u < units; u += kUnitSplit) {
+    // subset number (u + 1) / 2 of the bits of nzmask, and its source pattern
+    int S = 0;
+    {
+      uint32_t sub = (uint32_t)(u + 1) >> 1;
+      const uint32_t rev = u > 0 && (u & 1) == 0 ? ~0u : 0u;
+      int p3 = 1;
+      for (int b = 0; b < kb; ++b) {
+        if ((nzmask >> b) & 1u) {
+          if (sub & 1u) S += (1 + (((minus ^ rev) >> b) & 1u)) * p3;
+          sub >>= 1;
+        }
+        p3 *= 3;
+      }
+    }
+    const uint32_t lo = lstart[S] + (uint32_t)bz * (uint32_t)kChunk, s_end = lstart[S + 1];
+    if (lo >= s_end) continue;
+    const uint32_t hi = lo + kChunk < s_end ? lo + kChunk : s_end;
+    if (p_l1[lo] >= longest) continue;  // no source row of the chunk is shorter than any g
+    const bool open = mine && !dom[k];
+    if (!__any_sync(0xffffffffu, open)) return;
+    // the lanes of a warp read the same source rows at the same time: the loads are broadcasts
+    bool d = false;
+    if (open) {
+      if (u == 0)
+        d = scan_list<true, true>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
+      else if (u & 1)
+        d = scan_list<true, false>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
+      else
+        d = scan_list<false, true>(G, n, ldg, W, masks, lo, hi, k, gl1, np, nn, gsp, gsn, p_idx, p_pk, p_sig, p_l1);
+      if (d) dom[k] = 1;
+    }
+    __syncwarp();
+  }
 }
 
 __global__ void dominance_kernel(const int8_t* __restrict__ G, int n, int ldg, int W, const uint64_t* __restrict__ masks,
                                  const int4* __restrict__ gblk, const uint32_t* __restrict__ lstart, int kb,
                                  const uint32_t* __restrict__ p_idx, const uint64_t* __restrict__ p_pk,
                                  const ulonglong2* __restrict__ p_sig, const int32_t* __restrict__ p_l1,
-                                 uint8_t* __restrict__ dom) {
+                                 uint8_t* dom) {
   dominance_block(G, n, ldg, W, masks, gblk[blockIdx.x], lstart, kb, p_idx, p_pk, p_sig, p_l1, dom, blockIdx.y,
                   blockIdx.z);
 }
@@ -1245,7 +1265,7 @@ extern "C" int mape_minimal_filter(const int8_t* G, int64_t K, int32_t n, int32_
     }
     if (!gb.empty()) {
       MAPE_CUDA_TRY(cudaMemcpyAsync(gblk, gb.data(), sizeof(int4) * gb.size(), cudaMemcpyHostToDevice, st));
-      const dim3 grid((unsigned)gb.size(), 2u << kb, (unsigned)ceil_div(max_list, kChunk));
+      const dim3 grid((unsigned)gb.size(), kUnitSplit, (unsigned)ceil_div(max_list, kChunk));
       mape_detail::launch(dominance_kernel, grid, kTile, 0, st, G, n, ldg, W, masks, gblk, lstart, kb, p_idx, p_pk,
                           p_sig, p_l1, keep);
     }
@@ -1555,10 +1575,8 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
     // g-blocks of every instance: runs of at most kTile rows of one list
     std::vector<int4> gb;
     uint32_t max_list = 0;
-    int max_kb = 0;
     for (int i = 0; i < count; ++i) {
       if (v[(size_t)i].nvalid == 0) continue;
-      max_kb = std::max(max_kb, v[(size_t)i].kb);
       const std::vector<uint32_t>& l = lst[(size_t)i];
       for (int L = 0; L < v[(size_t)i].nlists; ++L) {
         const uint32_t a = l[(size_t)L], b = l[(size_t)L + 1];
@@ -1570,7 +1588,7 @@ extern "C" int mape_minimal_filter_batch(mape_minimal_item* items, int32_t count
     if (!gb.empty()) {
       if ((int64_t)gb.size() > gb_cap) return MAPE_ERR_CAPACITY;
       MAPE_CUDA_TRY(cudaMemcpyAsync(d_gblk, gb.data(), sizeof(int4) * gb.size(), cudaMemcpyHostToDevice, st));
-      const dim3 grid((unsigned)gb.size(), 2u << max_kb, (unsigned)ceil_div(max_list, kChunk));
+      const dim3 grid((unsigned)gb.size(), kUnitSplit, (unsigned)ceil_div(max_list, kChunk));
       launch(min_dominance_batch_kernel, grid, kTile, 0, st, cv_, (const int4*)d_gblk);
     }
   }
