@@ -1,6 +1,7 @@
-"""The kernel test over tiles of 32 transposed rows, and the route beside it
-(rows of A with a large absolute sum), against numpy in 64 bits at the edges of
-the tile, of its 16-byte pieces and of the packed 16-bit sums.  Integers: equal."""
+"""The kernel test and the coefficients over tiles of 32 transposed rows, and
+the routes beside them (rows of A with a large absolute sum; directions at any
+pitch), against numpy in 64 bits at the edges of the tile, of its 16-byte
+pieces, of the entry chunks and of the packed 16-bit sums.  Integers: equal."""
 import numpy as np
 import pytest
 
@@ -50,3 +51,27 @@ def test_kernel_test_tiles(M, m, n, K, big):
     want = np.all(G.astype(np.int64) @ A.T == 0, axis=1)
     ok, fails = M.kernel_test(dev(A.astype(np.int32)), dev(_pitched(M, G, n)), n)
     assert np.array_equal(ok.cpu().numpy().astype(bool), want) and fails == int((~want).sum())
+
+
+@pytest.mark.parametrize("n,K,nnz", [(1, 1, 1), (15, 31, 0), (16, 32, 100), (17, 33, 1023), (100, 64, 1024),
+                                     (1000, 70, 1025), (4096, 40, 5000)])
+@pytest.mark.parametrize("quartic,small", [(False, False), (True, False), (True, True)])
+@pytest.mark.parametrize("pitched", [True, False])
+def test_coeffs_tiles(M, n, K, nnz, quartic, small, pitched):
+    rng = np.random.default_rng(n + K + nnz)
+    G = rng.integers(-3, 4, size=(K, n))
+    G[:, 0] = -128
+    G[K // 2] = rng.choice([-128, 127], size=n)
+    G[0] = -128
+    qr = rng.integers(0, n, size=nnz).astype(np.int32)
+    qc = np.maximum(qr, rng.integers(0, n, size=nnz)).astype(np.int32)
+    # values at the ends of a chunk's 32-bit sums, and past them
+    qv = (rng.choice([-4095, 4095], size=nnz) if small else rng.integers(-2 ** 31, 2 ** 31, size=nnz)).astype(np.int32)
+    w = rng.integers(0, 2 ** 20, size=n).astype(np.int32) if quartic else None
+    g = G.astype(np.int64)
+    f = np.where(qr == qc, 1, 2) * qv.astype(np.int64)
+    want_a = (g[:, qr] * g[:, qc]) @ f if nnz else np.zeros(K, np.int64)
+    want_q = (g ** 4) @ w.astype(np.int64) if quartic else np.zeros(K, np.int64)
+    rows = _pitched(M, G, n) if pitched else G.astype(np.int8)
+    a, q4 = M.direction_coeffs(dev(qr), dev(qc), dev(qv), None if w is None else dev(w), n, dev(rows))
+    assert np.array_equal(a.cpu().numpy(), want_a) and np.array_equal(q4.cpu().numpy(), want_q)
