@@ -84,8 +84,8 @@ __global__ void kernel_test_kernel(const int32_t* __restrict__ A, int m, int n, 
 // warp per row of A.  When every row of A has sum |a| <= kTileSum they are
 // packed for the tile kernel (pack[q] = tile_at(column) | value << kTileShift,
 // start[r] = the sum's start, see there); else *big is set and they are col, val.
-// A row of a small sum (at most 255 entries, fewer than n) is filled up with
-// zero entries to a multiple of four.
+// A row of a small sum is filled up with zero entries to a multiple of four
+// (*big is set where that would take more than the n entries there is room for).
 constexpr int kTileSum = 255, kTileShift = 17;
 
 __global__ void csr_count_kernel(const int32_t* __restrict__ A, int m, int n, uint32_t* __restrict__ rowcnt,
@@ -105,8 +105,10 @@ __global__ void csr_count_kernel(const int32_t* __restrict__ A, int m, int n, ui
     sum += __shfl_xor_sync(0xffffffffu, sum, off);
   }
   if (lane == 0) {
-    rowcnt[r] = sum > kTileSum ? c : (c + 3) & ~3u;
-    if (sum > kTileSum) atomicOr(big, 1);
+    const uint32_t c4 = (c + 3) & ~3u;
+    const bool fits = sum <= kTileSum && c4 <= (uint32_t)n;
+    rowcnt[r] = fits ? c4 : c;
+    if (!fits) atomicOr(big, 1);
   }
 }
 

@@ -53,6 +53,23 @@ def test_kernel_test_tiles(M, m, n, K, big):
     assert np.array_equal(ok.cpu().numpy().astype(bool), want) and fails == int((~want).sum())
 
 
+@pytest.mark.parametrize("m,n", [(3100, 17), (3100, 16), (1600, 31), (800, 64)])
+def test_kernel_test_full_rows(M, m, n):
+    """Rows of A without zeros, where a fill to a multiple of four has no room."""
+    rng = np.random.default_rng(m + n)
+    A = np.tile(rng.choice([-2, -1, 1, 2], size=(1, n)), (m, 1))
+    A[m // 2:] *= -1
+    G = rng.integers(-3, 4, size=(70, n))
+    for k in range(0, 70, 2):      # an exact row: the last entries take up the sum
+        G[k, -2:] = 0
+        r = int(G[k] @ A[0])
+        G[k, -1] = -r // A[0, -1] if r % A[0, -1] == 0 else 0
+    want = np.all(G @ A.T == 0, axis=1)
+    assert want.any() and not want.all()
+    ok, fails = M.kernel_test(dev(A.astype(np.int32)), dev(_pitched(M, G, n)), n)
+    assert np.array_equal(ok.cpu().numpy().astype(bool), want) and fails == int((~want).sum())
+
+
 @pytest.mark.parametrize("n,K,nnz", [(1, 1, 1), (15, 31, 0), (16, 32, 100), (17, 33, 1023), (100, 64, 1024),
                                      (1000, 70, 1025), (4096, 40, 5000)])
 @pytest.mark.parametrize("quartic,small", [(False, False), (True, False), (True, True)])
