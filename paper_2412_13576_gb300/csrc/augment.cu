@@ -788,7 +788,7 @@ size_t score_smem(int n) {
 
 // the shared-memory limit of every variant, where it may take more than the default
 int allow_score_smem(size_t smem, bool batch) {
-  if (smem <= 48 * 1024) return MAPE_OK;
+  if (smem <= kSmemUnasked) return MAPE_OK;
   for (int lanes : kLaneChoices)
     for (bool vec : {true, false}) {
       if (!vec && lanes != 1) continue;
@@ -975,7 +975,7 @@ extern "C" int mape_direction_coeffs(const int32_t* q_row, const int32_t* q_col,
   if (ldg > kCoefMaxRow) return MAPE_ERR_SHAPE;
   if (ldg % 16 == 0 && (reinterpret_cast<uintptr_t>(G) & 15) == 0) {
     const size_t tile = tile_bytes(n) + sizeof(int4) * kCoefChunk;
-    if (tile > 48 * 1024) {
+    if (tile > kSmemUnasked) {
       size_t lim = 0;
       const int rc = allow_max_dynamic_smem((const void*)coeffs_tile_kernel, &lim);
       if (rc != MAPE_OK) return rc;

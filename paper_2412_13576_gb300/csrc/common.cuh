@@ -33,6 +33,11 @@ int allow_max_dynamic_smem(const void* func, size_t* limit);
 // Forgets the autotuned lane counts of Algorithm 1's scoring pass.
 void augment_tune_clear();
 
+// Dynamic shared memory that a launch may ask for without
+// allow_max_dynamic_smem: the 48 KB hold the kernel's static part too, at most
+// 8 KB in the kernels that are launched by this rule.
+constexpr size_t kSmemUnasked = 40 * 1024;
+
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

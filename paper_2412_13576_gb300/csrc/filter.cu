@@ -929,7 +929,7 @@ extern "C" int mape_kernel_test(const int32_t* A, int32_t m, int32_t n, const in
     mape_detail::launch(csr_fill_kernel, gw, 256, 0, st, A, m, n, rowptr, col, val, big, pack, rowcnt);
     // the device decides which of the two kernels works, the call does not wait for it
     const size_t tile = tile_bytes(n);
-    if (tile > 48 * 1024) {
+    if (tile > kSmemUnasked) {
       size_t lim = 0;
       const int rc = allow_max_dynamic_smem((const void*)kernel_test_tile_kernel, &lim);
       if (rc != MAPE_OK) return rc;

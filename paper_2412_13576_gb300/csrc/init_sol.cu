@@ -454,7 +454,7 @@ extern "C" int mape_initial_solutions(const mape_init_args* a, void* stream) {
   auto lists = n <= 128 ? init_sol_lists_kernel<1> : n <= 256 ? init_sol_lists_kernel<2>
              : n <= 512 ? init_sol_lists_kernel<4> : init_sol_lists_kernel<0>;
   const size_t lsm = (size_t)(n + m) * sizeof(float);
-  if (lsm > 48 * 1024) {
+  if (lsm > kSmemUnasked) {
     size_t lim = 0;
     const int rc = allow_max_dynamic_smem((const void*)lists, &lim);
     if (rc != MAPE_OK) return rc;

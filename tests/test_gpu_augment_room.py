@@ -40,7 +40,8 @@ def _best(G, a, r, x, l, u):
 
 @pytest.mark.parametrize("lanes", [1, 4, 32])
 @pytest.mark.parametrize("n,K,kind", [(1, 3, "few"), (15, 257, "all"), (16, 600, "all"), (17, 255, "extreme"),
-                                      (33, 1500, "few"), (130, 513, "extreme"), (4097, 300, "few")])
+                                      (33, 1500, "few"), (130, 513, "extreme"), (936, 300, "few"), (1212, 40, "few"),
+                                      (4097, 300, "few")])
 def test_unit_steps_and_queue(M, n, K, kind, lanes):
     rng = np.random.default_rng(n * 7 + K)
     span = 255 if kind == "extreme" else 3

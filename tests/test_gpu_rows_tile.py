@@ -27,7 +27,7 @@ def _pitched(M, G, n):
 
 
 @pytest.mark.parametrize("m,n,K", [(1, 257, 1), (33, 300, 31), (200, 260, 33), (5, 1000, 100), (70, 2500, 64),
-                                   (9, 4096, 65)])
+                                   (9, 4096, 65), (20, 1280, 40), (12, 1536, 33)])
 @pytest.mark.parametrize("big", [False, True])
 def test_kernel_test_tiles(M, m, n, K, big):
     rng = np.random.default_rng(m + n + K + big)
@@ -71,7 +71,7 @@ def test_kernel_test_full_rows(M, m, n):
 
 
 @pytest.mark.parametrize("n,K,nnz", [(1, 1, 1), (15, 31, 0), (16, 32, 100), (17, 33, 1023), (100, 64, 1024),
-                                     (1000, 70, 1025), (4096, 40, 5000)])
+                                     (1000, 70, 1025), (1024, 33, 500), (4096, 40, 5000)])
 @pytest.mark.parametrize("quartic,small", [(False, False), (True, False), (True, True)])
 @pytest.mark.parametrize("pitched", [True, False])
 def test_coeffs_tiles(M, n, K, nnz, quartic, small, pitched):
