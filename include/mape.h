@@ -627,7 +627,7 @@ int mape_set_allocator(mape_alloc_fn alloc_fn, mape_free_fn free_fn, void* ctx);
 
 /* Returns the memory the current device's library pool holds beyond what
  * live handles use (cudaMemPoolTrimTo(pool, 0) after a device
- * synchronisation).  OK when the pool was never created. */
+ * synchronisation) and destroys the streams kept of closed handles.  OK when the pool was never created. */
 int mape_trim_memory(void);
 
 typedef struct {

@@ -19,6 +19,7 @@
 #include <cstring>
 #include <mutex>
 #include <thread>
+#include <functional>
 #include <vector>
 
 namespace {
@@ -51,6 +52,37 @@ cudaMemPool_t library_pool(int dev) {
     g_pool[dev] = pool;
   }
   return g_pool[dev];
+}
+
+// Streams of closed handles, at most kIdleStreams per device, for the next
+// handles: a caching allocator keeps its free memory by stream, so a handle on a
+// stream of its own each time finds none of it (or another stream's, cold in
+// the TLBs).  Idle when they are put here; mape_trim_memory destroys them.
+constexpr size_t kIdleStreams = 16;
+std::mutex g_streams_mu;
+std::vector<cudaStream_t> g_streams[kMaxPoolDevices];
+
+cudaError_t take_stream(int dev, cudaStream_t* out) {
+  if (dev >= 0 && dev < kMaxPoolDevices) {
+    std::lock_guard<std::mutex> lk(g_streams_mu);
+    if (!g_streams[dev].empty()) {
+      *out = g_streams[dev].back();  // the last one closed
+      g_streams[dev].pop_back();
+      return cudaSuccess;
+    }
+  }
+  return cudaStreamCreateWithFlags(out, cudaStreamNonBlocking);
+}
+
+void give_stream(int dev, cudaStream_t st, bool idle) {
+  if (idle && dev >= 0 && dev < kMaxPoolDevices) {
+    std::lock_guard<std::mutex> lk(g_streams_mu);
+    if (g_streams[dev].size() < kIdleStreams) {
+      g_streams[dev].push_back(st);
+      return;
+    }
+  }
+  cudaStreamDestroy(st);
 }
 
 // A B = 0 exactly, row blockIdx.y of A against 128 columns of B: the row's
@@ -201,6 +233,27 @@ struct mape_instance {
     if (p) list.push_back({p, bytes});
     return static_cast<T*>(p);
   }
+  // Several buffers placed in one allocation, at 256-byte boundaries.  An
+  // allocation may be a call into the caller's allocator (the Python binding's
+  // takes the interpreter's lock, tens of microseconds each, one thread at a
+  // time): a handle's 33 allocations and as many releases were most of the time of 16
+  // requests at once, 57 ms; 28 with one per stage.
+  struct Buffers {
+    std::vector<std::pair<size_t, std::function<void(char*)>>> parts;
+    size_t bytes = 0;
+    template <typename T>
+    void add(T*& p, size_t count) {
+      p = nullptr;
+      parts.emplace_back(bytes, [&p](char* at) { p = reinterpret_cast<T*>(at); });
+      bytes += mape_detail::align_up(std::max<size_t>(16, count * sizeof(T)), 256);
+    }
+    bool place(mape_instance* h, std::vector<std::pair<void*, size_t>>& list) {
+      char* base = h->take<char>(list, bytes);
+      if (!base) return false;
+      for (auto& part : parts) part.second(base + part.first);
+      return true;
+    }
+  };
   void release_all(std::vector<std::pair<void*, size_t>>& list) {
     for (auto& pr : list) release(pr.first, pr.second);
     list.clear();
@@ -441,12 +494,13 @@ int set_objective(mape_instance* h, const mape_problem* f) {
     for (int i = 0; i < n; ++i)
       if (f->w[i] < 0) return MAPE_ERR_INVALID_ARG;
   h->nnz = (int)qv.size();
-  h->dqr = h->take<int32_t>(h->owned, qr.size());
-  h->dqc = h->take<int32_t>(h->owned, qc.size());
-  h->dqv = h->take<int32_t>(h->owned, qv.size());
-  h->dc = h->take<int32_t>(h->owned, n);
-  h->dw = h->take<int32_t>(h->owned, n);
-  if (!h->dqr || !h->dqc || !h->dqv || !h->dc || !h->dw) return MAPE_ERR_OOM;
+  mape_instance::Buffers bufs;
+  bufs.add(h->dqr, qr.size());
+  bufs.add(h->dqc, qc.size());
+  bufs.add(h->dqv, qv.size());
+  bufs.add(h->dc, n);
+  bufs.add(h->dw, n);
+  if (!bufs.place(h, h->owned)) return MAPE_ERR_OOM;
   H_TRY(upload(h, h->dqr, qr.data(), qr.size() * 4));
   H_TRY(upload(h, h->dqc, qc.data(), qc.size() * 4));
   H_TRY(upload(h, h->dqv, qv.data(), qv.size() * 4));
@@ -476,6 +530,12 @@ extern "C" int mape_set_allocator(mape_alloc_fn a, mape_free_fn f, void* ctx) {
 extern "C" int mape_trim_memory(void) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxPoolDevices) return MAPE_ERR_CUDA;
+  std::vector<cudaStream_t> idle_streams;
+  {
+    std::lock_guard<std::mutex> lk(g_streams_mu);
+    idle_streams.swap(g_streams[dev]);
+  }
+  for (cudaStream_t st : idle_streams) cudaStreamDestroy(st);
   cudaMemPool_t pool = nullptr;
   {
     std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -514,7 +574,7 @@ extern "C" int mape_create_instance(const int32_t* A, const int64_t* b, const in
   if (stream) {
     h->stream = mape_detail::as_stream(stream);
   } else {
-    if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) { delete h; return MAPE_ERR_CUDA; }
+    if (take_stream(h->dev, &h->stream) != cudaSuccess) { delete h; return MAPE_ERR_CUDA; }
     h->own_stream = true;
   }
   auto fail = [&](int rc) {
@@ -522,14 +582,16 @@ extern "C" int mape_create_instance(const int32_t* A, const int64_t* b, const in
     return rc;
   };
   const int d = h->d;
-  h->dA = h->take<int32_t>(h->owned, (size_t)m * n);
-  h->dB = h->take<int32_t>(h->owned, (size_t)n * d);
-  h->db = h->take<int64_t>(h->owned, (size_t)m);
-  h->dl = h->take<int32_t>(h->owned, n);
-  h->du = h->take<int32_t>(h->owned, n);
-  h->dspan = h->take<int32_t>(h->owned, n);
-  int32_t* dbad = h->take<int32_t>(h->owned, 1);
-  if (!h->dA || !h->dB || !h->db || !h->dl || !h->du || !h->dspan || !dbad) return fail(MAPE_ERR_OOM);
+  int32_t* dbad = nullptr;
+  mape_instance::Buffers bufs;
+  bufs.add(h->dA, (size_t)m * n);
+  bufs.add(h->dB, (size_t)n * d);
+  bufs.add(h->db, (size_t)m);
+  bufs.add(h->dl, n);
+  bufs.add(h->du, n);
+  bufs.add(h->dspan, n);
+  bufs.add(dbad, 1);
+  if (!bufs.place(h, h->owned)) return fail(MAPE_ERR_OOM);
   std::vector<int32_t> span(n);
   for (int i = 0; i < n; ++i) span[i] = u[i] - l[i];
   int rc;
@@ -587,28 +649,28 @@ int prepare_job(mape_handle h, int32_t P, const float* Z0, const float* G0) {
   cap = std::max<int64_t>(cap, (int64_t)P + 1);
   h->cap = cap;
   h->P = P;
-  h->dZ = h->take<float>(h->job_bufs, (size_t)P * d);
-  h->dM = h->take<float>(h->job_bufs, (size_t)P * d);
-  h->dV = h->take<float>(h->job_bufs, (size_t)P * d);
-  h->dG0 = G0 ? h->take<float>(h->job_bufs, (size_t)P * n) : nullptr;
-  h->dBuf0 = h->take<int8_t>(h->job_bufs, (size_t)cap * ldg);
-  h->dBuf1 = h->take<int8_t>(h->job_bufs, (size_t)cap * ldg);
-  h->dOk = h->take<uint8_t>(h->job_bufs, (size_t)cap);
-  h->dKeep = h->take<uint8_t>(h->job_bufs, (size_t)cap);
-  h->da = h->take<int64_t>(h->job_bufs, (size_t)cap);
-  h->dq4 = h->take<int64_t>(h->job_bufs, (size_t)cap);
-  h->dCount = h->take<unsigned long long>(h->job_bufs, 1);
-  h->dFlags = h->take<int32_t>(h->job_bufs, 1);
+  mape_instance::Buffers bufs;
+  bufs.add(h->dZ, (size_t)P * d);
+  bufs.add(h->dM, (size_t)P * d);
+  bufs.add(h->dV, (size_t)P * d);
+  h->dG0 = nullptr;
+  if (G0) bufs.add(h->dG0, (size_t)P * n);
+  bufs.add(h->dBuf0, (size_t)cap * ldg);
+  bufs.add(h->dBuf1, (size_t)cap * ldg);
+  bufs.add(h->dOk, (size_t)cap);
+  bufs.add(h->dKeep, (size_t)cap);
+  bufs.add(h->da, (size_t)cap);
+  bufs.add(h->dq4, (size_t)cap);
+  bufs.add(h->dCount, 1);
+  bufs.add(h->dFlags, 1);
   size_t w = 0;
   w = std::max(w, mape_extract_workspace_bytes(n, d, P, h->cfg.precision));
   w = std::max(w, mape_dedup_workspace_bytes(cap, ldg));
   w = std::max(w, mape_kernel_test_workspace_bytes(h->m, n));
   w = std::max(w, mape_minimal_workspace_bytes(cap, n));
   h->work_bytes = w;
-  h->dWork = h->take<char>(h->job_bufs, w);
-  if (!h->dZ || !h->dM || !h->dV || (G0 && !h->dG0) || !h->dBuf0 || !h->dBuf1 || !h->dOk ||
-      !h->dKeep || !h->da || !h->dq4 || !h->dCount || !h->dFlags || !h->dWork)
-    return MAPE_ERR_OOM;
+  bufs.add(h->dWork, w);
+  if (!bufs.place(h, h->job_bufs)) return MAPE_ERR_OOM;
   int rc = G0 ? upload(h, h->dG0, G0, sizeof(float) * (size_t)P * n) : upload(h, h->dZ, Z0, sizeof(float) * (size_t)P * d);
   if (rc) return rc;
   MAPE_CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -814,12 +876,14 @@ int prepare_augment(mape_handle h, const int32_t* X0, int32_t S, const mape_prob
   const int n = h->n;
   h->release_all(h->aug_bufs);
   h->S = S;
-  h->dX = h->take<int32_t>(h->aug_bufs, (size_t)S * n);
-  h->dF = h->take<int64_t>(h->aug_bufs, (size_t)S);
-  int32_t* dbad = h->take<int32_t>(h->aug_bufs, 1);
   h->aug_work_bytes = mape_augment_workspace_bytes(n, S, h->K);
-  h->dAugWork = h->take<char>(h->aug_bufs, h->aug_work_bytes);
-  if (!h->dX || !h->dF || !dbad || !h->dAugWork) return MAPE_ERR_OOM;
+  int32_t* dbad = nullptr;
+  mape_instance::Buffers bufs;
+  bufs.add(h->dX, (size_t)S * n);
+  bufs.add(h->dF, (size_t)S);
+  bufs.add(dbad, 1);
+  bufs.add(h->dAugWork, h->aug_work_bytes);
+  if (!bufs.place(h, h->aug_bufs)) return MAPE_ERR_OOM;
   int rc = upload(h, h->dX, X0, sizeof(int32_t) * (size_t)S * n);
   if (rc) return rc;
   MAPE_CUDA_TRY(cudaMemsetAsync(dbad, 0, 4, h->stream));
@@ -1124,7 +1188,7 @@ extern "C" void mape_destroy(mape_handle h) {
   h->release_all(h->aug_bufs);
   h->release_all(h->job_bufs);
   h->release_all(h->owned);
-  if (h->stream) cudaStreamSynchronize(h->stream);
-  if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
+  const cudaError_t e = h->stream ? cudaStreamSynchronize(h->stream) : cudaSuccess;
+  if (h->own_stream && h->stream) give_stream(h->dev, h->stream, e == cudaSuccess);
   delete h;
 }
