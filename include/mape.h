@@ -309,7 +309,7 @@ int mape_dedup_static(const int8_t* cand, int64_t count, int32_t n, int32_t ldc,
  * item i is one mape_dedup call -- its own rows, count, n, ldc, output and
  * workspace of mape_dedup_workspace_bytes(count, ldc) -- and gets the same
  * output and K.  Every kernel of the stage runs once over the rows of all
- * sets (hash, insert, compaction, keys, the bitonic stages, the run sorts,
+ * sets (hash, insert, compaction, keys, the sorted tiles, the merge passes,
  * the gather), each thread, warp or block finding its set by binary search
  * over the launch's prefix table; `workspace` holds the batch's tables
  * (mape_dedup_batch_workspace_bytes(count)).  Per item: K (distinct rows)
