@@ -664,8 +664,8 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
       const bool dbg = s == 0 && (p.dbg_phi || p.dbg_grad);
       const bool inv_on = inv_term != 0.f;
       // z of this thread's coordinates as the last step left it (at the first
-      // step, of all the start's)
-      const bool slow = __any_sync(0xffffffffu, p.eps < 1e-15f || (s == 0 ? zinf : zmost) >= kRintMost / 2);
+      // step, of all the start's, where a NaN in coordinate 0 hides the others)
+      const bool slow = __any_sync(0xffffffffu, p.eps < 1e-15f || !((s == 0 ? zinf : zmost) < kRintMost / 2));
       float nzinf = 0.f, frac = 0.f, l1_id = 0.f;
       float dsum = 0.f;  // sum of |rint(z_new) - rint(z_old)|: 0 iff no rounding changed
       int nkmax = -1, first_id = kNoNz;  // the first maximiser of |z|; the first nonzero rounding
