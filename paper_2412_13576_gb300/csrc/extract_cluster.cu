@@ -38,6 +38,7 @@
 // bits.
 #include "common.cuh"
 #include "extract_internal.cuh"
+#include "refill_stage.cuh"
 #include "tc_ptx.cuh"
 
 #include <algorithm>
@@ -357,21 +358,35 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
     mma_commit_if(lead, accr);
     return true;
   };
-  // a time-out: the block's remaining steps only take part in the barriers
+  // A time-out: the phase ends for every warp at its next vote (wait_acc) or
+  // wait, and the block's remaining steps only take part in the barriers.  A warp
+  // leaves its chunks after the one whose wait ran out (what it computed of
+  // that one is void, as the flagged call is; refusing it before the stores
+  // cost 2 to 3% of every step).
   auto give_up = [&]() {
     *(volatile int*)&s_abort = 1;
     atomicOr(p.flags, 16);
   };
   // Every thread: the accumulator is ready.  Only warp 0 polls; the others
   // sleep at a block barrier (polled by all, they took the issue slots and the
-  // shared-memory queue from the two warps that feed the MMAs).
-  auto wait_acc = [&]() -> bool {
-    bool ok = true;
-    if (uwarp == 0) ok = mbar_wait_bounded(accr, accph);
+  // shared-memory queue from the two warps that feed the MMAs).  going: false
+  // for a warp whose own wait ran out; the answer is the same for every thread.
+  auto wait_acc = [&](bool going) -> bool {
+    bool ok = going;
+    if (uwarp == 0 && ok) ok = mbar_wait_bounded(accr, accph);
     accph ^= 1;
     const bool bad = __syncthreads_or(!ok) != 0;
     tc_fence_after();
     return !bad;
+  };
+  // a wait of the epilogue: another warp's time-out ends it, too
+  auto wait_or_abort = [&](uint32_t bar, uint32_t parity) -> bool {
+    if (mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    do {
+      if (mbar_try_wait(bar, parity)) return true;
+    } while (*(volatile int*)&s_abort == 0 && clock64() - t0 < kWaitCycles);
+    return false;
   };
   // The state of chunk ch (8 coordinates: 3 x 4 KB, contiguous in the blocked
   // arrays) into its stage, by one lane of the calling warp
@@ -431,9 +446,11 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
     if (rank == 0 && h == 0 && do_fwd) p.zkey[((s + 1) & 1) * P2 + pg] = 0ull;  // the next step's maximum
     float l1 = 0.f;
     bool out = false;
+    bool acc_ok = true;  // the same for every thread
 #pragma unroll 1
-    for (int rb = 0; rb < RS; rb += kRowBlk) {
+    for (int rb = 0; rb < RS && acc_ok; rb += kRowBlk) {
       const int N = RS - rb < kRowBlk ? RS - rb : kRowBlk;
+      bool ok = true;
       if (uwarp < 2 && !dead) {
         const bool f16 = do_fwd && !p.f8, f8 = do_fwd && p.f8;
         // a stage holds its chunks' z (hi, lo, round(z)), then Bm, then Bm in e4m3
@@ -444,7 +461,6 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
         const uint32_t bytes = zb + rb16 + b16 + b8;
         int grp, nst;
         geometry(bytes, ring_fwd, grp, nst);
-        bool ok;
         if (uwarp == 1) {
           fence_async_all();
           const uint8_t* bf = p.Bf + ((size_t)(row0 + rb) * p.d32) * 2;
@@ -513,7 +529,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
       }
       __syncwarp();
       if (!dead) {
-        const bool acc_ok = wait_acc();
+        acc_ok = wait_acc(ok);
         // the ring is free: the first chunks of the state are on their way
         // before the gradient is
         if (do_fwd && (uwarp == 0 || uwarp == 4) && acc_ok && rb + kRowBlk >= RS) prefetch_state();
@@ -575,7 +591,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
     dead = __syncthreads_or(*(volatile int*)&s_abort) != 0;
 
     // ---- gradient ----
-    auto issue_grad = [&](int cb) {  // warps 0 and 1
+    auto issue_grad = [&](int cb) -> bool {  // warps 0 and 1
       const int N = CS - cb < kColBlk ? CS - cb : kColBlk;
       const uint32_t nb = (uint32_t)N * kKC * 2;
       int grp, nst;
@@ -608,10 +624,12 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
       }
       if (!ok) give_up();
       __syncwarp();
+      return ok;
     };
+    bool ok = true;  // no wait of this warp has run out
     if (do_fwd && uwarp < 2 && !dead && CS > 0) {
       if (uwarp == 1) fence_async_all();
-      issue_grad(0);
+      ok = issue_grad(0);
     }
     __syncwarp();
     // the candidates of step s - 1, the starts spread over the cluster's blocks
@@ -669,15 +687,15 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
       float nzinf = 0.f, frac = 0.f, l1_id = 0.f;
       float dsum = 0.f;  // sum of |rint(z_new) - rint(z_old)|: 0 iff no rounding changed
       int nkmax = -1, first_id = kNoNz;  // the first maximiser of |z|; the first nonzero rounding
-      bool out_id = false, nan_head = false, ok = true;
+      bool out_id = false, nan_head = false;
       int8_t* srow = p.stage + (((s + 1) & 1) * P2 + pg) * p.lds;
 #pragma unroll 1
-      for (int cb = 0; cb < CS && ok; cb += kColBlk) {
+      for (int cb = 0; cb < CS; cb += kColBlk) {
         const int nch = (CS - cb < kColBlk ? CS - cb : kColBlk) / 8;
-        if (cb > 0 && uwarp < 2) issue_grad(cb);
+        if (cb > 0 && uwarp < 2 && ok) ok = issue_grad(cb);
         __syncwarp();
-        ok = wait_acc();
-        if (!ok) {
+        if (!wait_acc(ok)) {  // every warp leaves here
+          ok = false;
           if (tid == 0) give_up();
           break;
         }
@@ -686,7 +704,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
           uint32_t gv[8];
           tmem_ld8(tmem + lane_base + ch * 8, gv);
           const uint32_t e = ec + (uint32_t)(cb / 8 + ch), st = e % kEStages;
-          if (!mbar_wait_bounded(efull0 + 8 * st, (e / kEStages) & 1u)) ok = false;
+          if (!wait_or_abort(efull0 + 8 * st, (e / kEStages) & 1u)) ok = false;
           const float4* es = reinterpret_cast<const float4*>(smem + ering0 + st * kEBytes) + r;
           const float4 cz[2] = {es[0], es[kTM]}, cm[2] = {es[2 * kTM], es[3 * kTM]}, cv[2] = {es[4 * kTM], es[5 * kTM]};
           float zc[8] = {cz[0].x, cz[0].y, cz[0].z, cz[0].w, cz[1].x, cz[1].y, cz[1].z, cz[1].w};
@@ -823,18 +841,19 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
           }
           // the stage's next chunk, once the three other warps have read it
           if (q == 0 && cb / 8 + ch + kEStages < CS / 8) {
-            if (!mbar_wait_bounded(eempty0 + 8 * st, (e / kEStages) & 1u)) ok = false;
-            __syncwarp();
-            load_state(cb / 8 + ch + kEStages);
+            ok = mape_detail::refill_stage(
+                ok, [&] { return wait_or_abort(eempty0 + 8 * st, (e / kEStages) & 1u); },
+                [](bool b) { return __all_sync(0xffffffffu, b) != 0; }, [&] { load_state(cb / 8 + ch + kEStages); });
             __syncwarp();
           }
         };
 #pragma unroll 1
-        for (int ch = h; ch < nch; ch += 2) chunk(ch);
-        if (!__all_sync(0xffffffffu, ok)) {
-          if (lane == 0) give_up();
-          ok = true;  // the blocks' barriers are still to be met by every warp
+        for (int ch = h; ch < nch; ch += 2) {
+          chunk(ch);
+          if (!__all_sync(0xffffffffu, ok)) break;
         }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok && lane == 0) give_up();
         tc_fence_before();
         __syncwarp();
         if (lane == 0 && cb + kColBlk < CS) mbar_arrive(accf);
