@@ -30,7 +30,13 @@
 // piece that rules it out; the directions that remain are queued in shared
 // memory, and full blocks of them get their partial sums (exact int64) and
 // lambda bounds, combined by shuffles.  45 000 directions of n = 200, 64 starts:
-// 0.48 ms an iteration before, 0.16 now.
+// 0.48 ms an iteration without it, 0.14 with it.  Where most directions have
+// room (wide boxes) it is pure addition: every pass counts them, and the next
+// one asks first only while they were at most a quarter (a test of all costs
+// 0.45 to 0.75 of the sums, dense and sparse rows; the first pass goes by a
+// sample).  60 passes of the same size, all with room, dense and sparse rows:
+// 49.3 and 30.1 ms without the test, 76.1 and 49.2 with it, 50.4 and 28.9 by
+// this rule.
 //
 // Many instances at once (mape_augment_run_batch): one score and one apply
 // launch per iteration cover the starts of every instance, each block finding
@@ -279,21 +285,61 @@ struct AugView {
   long long* R;
   uint8_t* active;
   Best* partial;
+  // [S] each: directions with room for a unit step by the last pass, the same in
+  // this one, rounds that this one has handed to its blocks
+  unsigned long long *fit, *fit_now, *next;
   int32_t* iters;
   unsigned int* n_active;
   int32_t* bad;
   int64_t max_iters;
 };
 
+// the pre-pass: where its tables fit beside the others in shared memory
+__host__ __device__ inline bool score_pre(int n) { return n <= 4096; }
+
 constexpr int kScoreThreads = 256;
-constexpr int kMaxScoreBlocks = 1024;  // per start
-constexpr int kScoreBlocks = 1216;     // of a launch over all starts: 8 per SM, each staging its start's tables once
+constexpr int kMaxPartials = 1024;                 // per start, the last two for its three counters
+constexpr int kMaxScoreBlocks = kMaxPartials - 2;  // per start
+// of a launch over all starts, each staging its start's tables: 16 per SM, of
+// which 4 or 5 run at once (8 per SM: 1 to 10% slower passes, the last blocks
+// alone on the chip; 64 per SM: 10% slower with the pre-pass, for the staging)
+constexpr int kScoreBlocks = 2432;
 
 // One block per start, bound by the latency of its passes over Q: 1024 threads
 // and several entries of each in flight (256 threads, an entry at a time: 143 us
 // on average for 16 instances of up to 1500 variables, 62 now; the
 // apply pass, which changes r only where the move is not zero, 9.2 and 5.9).
 constexpr int kStartThreads = 1024;
+
+// Directions of start s with room for a unit step at x, estimated from 32 of
+// them spread over the set, one per warp: the first pass's choice between its
+// two forms.
+static_assert(kStartThreads == 32 * 32);
+
+__device__ __forceinline__ void sample_fit(const AugView& v, int s) {
+  const int32_t* x = v.X + (int64_t)s * v.n;
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = threadIdx.x >> 5;
+  const bool mine = warp < v.K;
+  const int8_t* g = v.G + (v.K < 32 ? (mine ? warp : 0) : (warp * v.K) >> 5) * v.ldg;
+  bool plus = mine, minus = mine;  // the same for the warp
+  for (int i0 = 0; i0 < v.n && (plus || minus); i0 += 32) {
+    const int i = i0 + lane;
+    bool p = true, m = true;
+    if (i < v.n) {
+      const int gi = g[i], xi = x[i], up = v.u[i] - xi, dn = xi - v.l[i];
+      p = gi <= up && -gi <= dn;
+      m = gi <= dn && -gi <= up;
+    }
+    plus = __all_sync(0xffffffffu, p) && plus;
+    minus = __all_sync(0xffffffffu, m) && minus;
+  }
+  const int fits = __syncthreads_count(lane == 0 && (plus || minus));
+  if (threadIdx.x == 0) {
+    v.fit[s] = v.K < 32 ? (unsigned long long)fits : (unsigned long long)(fits * v.K) >> 5;
+    v.fit_now[s] = 0;
+  }
+}
 
 // r = 2 Q x + c and f(x) of start s; checks l <= x <= u.
 __device__ __forceinline__ void init_body(const AugView& v, int s) {
@@ -328,7 +374,9 @@ __device__ __forceinline__ void init_body(const AugView& v, int s) {
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += s_f[i];
     v.fval[s] = t;
     v.active[s] = 1;
+    v.next[s] = 0;
   }
+  if (score_pre(v.n)) sample_fit(v, s);
 }
 
 __device__ __forceinline__ long long floor_div(long long a, long long b) {  // b > 0
@@ -339,14 +387,17 @@ __device__ __forceinline__ long long floor_div(long long a, long long b) {  // b
 
 // The per-start tables the score pass reads for every direction, by
 // coordinate i: rw[2 i] = (r_i, w x_i^3), rw[2 i + 1] = (w x_i^2, w x_i) with
-// r = 2 Q x + c (the w terms 0 without the quartic term), ud[i] = (u - x,
-// x - l), so that an entry takes one 16-byte load (two with the quartic term)
-// and one 8-byte load.
+// r = 2 Q x + c, ud[i] = (u - x, x - l), so that an entry takes one 16-byte
+// load (two with the quartic term) and one 8-byte load.  Without the quartic
+// term rw[i] = (r_i, 0): what the tables leave of the SM is the L1 that holds
+// the rows' lines between the pieces of a thread (60 passes of 4 starts over
+// 50 000 sparse directions of 2000 entries: 25.7 ms with 80 KB of tables a
+// block, 29.7 with 100, 17.4 with the 66 now).
 struct ScoreSmem {
   longlong2* rw;
   int2* ud;
   const uint4* room;    // two per word of 4 coordinates (room_fits; with the pre-pass only)
-  int64_t* queue;       // 2 kScoreThreads directions (with the pre-pass only)
+  uint32_t* queue;      // 2 kScoreThreads directions, numbered within the block (with the pre-pass only)
   const uint32_t* rcp;  // rcp[b] = ceil(2^20 / b), b = 1 .. 128
 };
 
@@ -367,9 +418,6 @@ __device__ __forceinline__ void room_fits(uint32_t g4, const uint4 hi, const uin
 
 __host__ __device__ inline int score_words(int n) { return (n + 15) / 16 * 4; }
 
-// the pre-pass: where its tables fit beside the others in shared memory
-__host__ __device__ inline bool score_pre(int n) { return n <= 4096; }
-
 // floor(a / b) for 0 <= a < 2048 and 1 <= b <= 128 as (a ceil(2^20 / b)) >> 20:
 // with ceil(2^20 / b) = (2^20 + e) / b, 0 <= e < b, the product is
 // 2^20 (a / b) + a e / b and a e < 2^20, so the shift drops only the fraction
@@ -382,16 +430,18 @@ __device__ __forceinline__ int div_small(int a, int b, const uint32_t* rcp) {
   return a / b;
 }
 
-__device__ __forceinline__ ScoreSmem stage_start(const AugView& v, int s) {
+template <bool kQuartic>
+__device__ __forceinline__ ScoreSmem stage_start(const AugView& v, int s, bool pre) {
   extern __shared__ __align__(16) long long smem[];
   const int n = v.n;
   ScoreSmem t;
-  t.rw = reinterpret_cast<longlong2*>(smem);                 // 32 n bytes
+  constexpr int rs = kQuartic ? 2 : 1;
+  t.rw = reinterpret_cast<longlong2*>(smem);                      // 16 rs n bytes
   const int nw = score_words(n);
-  t.ud = reinterpret_cast<int2*>(smem + 4 * (int64_t)n);     // 8 n bytes
-  uint4* room = reinterpret_cast<uint4*>(smem + 5 * (int64_t)n + (n & 1));  // 32 bytes per word
+  t.ud = reinterpret_cast<int2*>(smem + 2 * rs * (int64_t)n);     // 8 n bytes
+  uint4* room = reinterpret_cast<uint4*>(smem + (2 * rs + 1) * (int64_t)n + (n & 1));  // 32 bytes per word
   t.room = room;
-  t.queue = reinterpret_cast<int64_t*>(room + 2 * (int64_t)nw);
+  t.queue = reinterpret_cast<uint32_t*>(room + 2 * (int64_t)nw);
   __shared__ uint32_t s_rcp[129];
   for (int b = threadIdx.x; b <= 128; b += blockDim.x)
     s_rcp[b] = b ? ((1u << kRcpShift) + (uint32_t)b - 1u) / (uint32_t)b : 0u;
@@ -399,12 +449,17 @@ __device__ __forceinline__ ScoreSmem stage_start(const AugView& v, int s) {
   const int32_t* x = v.X + (int64_t)s * n;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const long long xi = x[i];
-    const long long wi = v.w ? v.w[i] : 0;
-    t.rw[2 * i] = make_longlong2(v.R[(int64_t)s * n + i], wi * xi * xi * xi);
-    t.rw[2 * i + 1] = make_longlong2(wi * xi * xi, wi * xi);
+    const long long ri = v.R[(int64_t)s * n + i];
+    if (kQuartic) {
+      const long long wi = v.w[i];
+      t.rw[2 * i] = make_longlong2(ri, wi * xi * xi * xi);
+      t.rw[2 * i + 1] = make_longlong2(wi * xi * xi, wi * xi);
+    } else {
+      t.rw[i] = make_longlong2(ri, 0);
+    }
     t.ud[i] = make_int2(v.u[i] - x[i], x[i] - v.l[i]);
   }
-  for (int w = threadIdx.x; score_pre(n) && w < nw; w += blockDim.x) {
+  for (int w = threadIdx.x; pre && w < nw; w += blockDim.x) {
     uint32_t hi[2][2] = {{0, 0}, {0, 0}}, lo[2][2] = {{0, 0}, {0, 0}};  // [up, down][even, odd]
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
@@ -433,10 +488,11 @@ struct DirSums {
   int lam_p = 0x7fffffff, lam_m = 0x7fffffff;  // lambda_max for +g and -g
 };
 
-__device__ __forceinline__ void add_entry(DirSums& d, const ScoreSmem& t, bool quartic, int i, int gi) {
-  const longlong2 rw = t.rw[2 * i];
+template <bool kQuartic>
+__device__ __forceinline__ void add_entry(DirSums& d, const ScoreSmem& t, int i, int gi) {
+  const longlong2 rw = t.rw[kQuartic ? 2 * i : i];
   d.b += (long long)gi * rw.x;
-  if (quartic) {  // g^2 <= 2^14 and |g^3| <= 2^21: one 64 x 32-bit product each
+  if (kQuartic) {  // g^2 <= 2^14 and |g^3| <= 2^21: one 64 x 32-bit product each
     const longlong2 ww = t.rw[2 * i + 1];
     const int g2 = gi * gi;
     d.c1 += rw.y * gi;
@@ -451,15 +507,16 @@ __device__ __forceinline__ void add_entry(DirSums& d, const ScoreSmem& t, bool q
 }
 
 // The best move along +-g_k given the direction's sums.
+template <bool kQuartic>
 __device__ __forceinline__ void best_move(const AugView& v, int64_t k, const DirSums& d, Best& best) {
   long long ak = v.a[k];
-  long long c4 = v.q4[k];
+  const long long c4 = kQuartic ? v.q4[k] : 0;
   for (int e = 1; e >= -1; e -= 2) {
     int L = (e > 0) ? d.lam_p : d.lam_m;
     // L <= max(u - l) <= 127 for a nonzero row; a zero row has no move
     if (L < 1 || L > 255) continue;
     long long eb = e * d.b;
-    if (!v.w) {
+    if (!kQuartic) {
       long long cand[2];
       if (ak > 0) {
         // vertex at -eb / (2 a); the integer minimiser is floor or ceil of it
@@ -491,15 +548,17 @@ __device__ __forceinline__ void best_move(const AugView& v, int64_t k, const Dir
 // Score block bx of start s.  kL lanes per direction; kVec: the rows are read
 // as 16-byte pieces (ldg a multiple of 16, G 16-byte aligned), else byte by
 // byte (kL = 1).
-template <int kL, bool kVec>
+template <int kL, bool kVec, bool kQuartic>
 __device__ __forceinline__ void score_body(const AugView& v, int s, int bx) {
   if (!v.active[s]) return;  // block-uniform
-  const ScoreSmem t = stage_start(v, s);
-  __syncthreads();
   const int n = v.n;
-  const bool quartic = v.w != nullptr;
+  // with the pre-pass while at most a quarter of the directions had room
+  const bool pre = kVec && score_pre(n) && 4 * v.fit[s] <= (unsigned long long)v.K;
+  const ScoreSmem t = stage_start<kQuartic>(v, s, pre);
+  __syncthreads();
+  unsigned fit = 0;  // of the directions this thread has tested
   const int sub = threadIdx.x % kL;
-  const int per_block = blockDim.x / kL;  // directions per block and round
+  constexpr int per_block = kScoreThreads / kL;  // directions per block and round
   Best best{kNoMove, kNoMove};
   // the sums and bounds of direction k (k < 0: none), by its group of lanes
   auto score = [&](int64_t k) {
@@ -514,13 +573,13 @@ __device__ __forceinline__ void score_body(const AugView& v, int s, int bx) {
           for (int b = 0; b < 16; ++b) {
             const int i = p * 16 + b;
             const int gi = (int)(int8_t)(w4[b >> 2] >> (8 * (b & 3)));
-            if (gi != 0 && i < n) add_entry(d, t, quartic, i, gi);
+            if (gi != 0 && i < n) add_entry<kQuartic>(d, t, i, gi);
           }
         }
       } else {
         for (int i = 0; i < n; ++i) {
           const int gi = g[i];
-          if (gi != 0) add_entry(d, t, quartic, i, gi);
+          if (gi != 0) add_entry<kQuartic>(d, t, i, gi);
         }
       }
     }
@@ -528,78 +587,96 @@ __device__ __forceinline__ void score_body(const AugView& v, int s, int bx) {
 #pragma unroll
       for (int o = kL / 2; o > 0; o >>= 1) {
         d.b += __shfl_xor_sync(0xffffffffu, d.b, o);
-        d.c1 += __shfl_xor_sync(0xffffffffu, d.c1, o);
-        d.c2 += __shfl_xor_sync(0xffffffffu, d.c2, o);
-        d.c3 += __shfl_xor_sync(0xffffffffu, d.c3, o);
+        if (kQuartic) {
+          d.c1 += __shfl_xor_sync(0xffffffffu, d.c1, o);
+          d.c2 += __shfl_xor_sync(0xffffffffu, d.c2, o);
+          d.c3 += __shfl_xor_sync(0xffffffffu, d.c3, o);
+        }
         d.lam_p = min(d.lam_p, __shfl_xor_sync(0xffffffffu, d.lam_p, o));
         d.lam_m = min(d.lam_m, __shfl_xor_sync(0xffffffffu, d.lam_m, o));
       }
     }
-    if (k >= 0 && sub == 0) best_move(v, k, d, best);
+    if (k >= 0 && sub == 0) {
+      if (kVec && !pre) fit += d.lam_p >= 1 || d.lam_m >= 1;
+      best_move<kQuartic>(v, k, d, best);
+    }
   };
-  if (!kVec) {
-    for (int64_t k0 = (int64_t)bx * per_block; k0 < v.K; k0 += (int64_t)v.nb * per_block) {  // block-uniform
-      const int64_t k = k0 + threadIdx.x;
+  if (!kVec || !pre) {
+    // A round's directions are scored as they come.  Where a block has several
+    // rounds, it takes the start's next one when it is ready: with a fixed share
+    // SMs were idle at the end of a pass (64 starts, 45 000 dense directions of
+    // 200 entries with room, 60 passes: 51.2 ms, 50.4 now; quartic 79.5 and 77.0).
+    __shared__ unsigned long long s_round;
+    const bool several = (int64_t)v.nb * per_block < v.K;
+    for (int64_t round = bx;;) {  // block-uniform
+      if (several) {
+        if (threadIdx.x == 0) s_round = atomicAdd(&v.next[s], 1ull);
+        __syncthreads();
+        round = (int64_t)s_round;
+        __syncthreads();
+      }
+      const int64_t k0 = round * per_block;
+      if (k0 >= v.K) break;
+      const int64_t k = k0 + threadIdx.x / kL;
       score(k < v.K ? k : -1);
+      if (!several) break;
     }
   } else {
-    // with the pre-pass the directions that remain go through the queue (two
-    // blocks of them at most); without it (score_pre) a round's directions are scored as they come
-    const bool pre = score_pre(n);
+    // the directions that remain go through the queue (two blocks of them at most)
     __shared__ int s_queued;
     if (threadIdx.x == 0) s_queued = 0;
     __syncthreads();
-    for (int64_t k0 = (int64_t)bx * per_block;; k0 += (int64_t)v.nb * per_block) {  // block-uniform
+    uint32_t first = 0;  // directions of the block's earlier rounds (K < 2^32 nb: a row has 16 bytes)
+    for (int64_t k0 = (int64_t)bx * per_block;; k0 += (int64_t)v.nb * per_block, first += per_block) {  // block-uniform
       const bool last = k0 >= v.K;
-      int cnt = last ? 0 : per_block;
-      if (pre) {
-        const int64_t k = k0 + threadIdx.x / kL;
-        uint32_t plus = k < v.K ? kBit8 : 0u, minus = plus;
-        if (k < v.K) {
-          const int8_t* g = v.G + k * v.ldg;
-          for (int p = sub; p * 16 < n; p += kL) {
-            const uint4 q = *reinterpret_cast<const uint4*>(g + p * 16);
-            const uint4* room = t.room + 8 * p;
-            room_fits(q.x, room[0], room[1], plus, minus);
-            room_fits(q.y, room[2], room[3], plus, minus);
-            room_fits(q.z, room[4], room[5], plus, minus);
-            room_fits(q.w, room[6], room[7], plus, minus);
-            if ((plus & kBit8) != kBit8 && (minus & kBit8) != kBit8) break;
-          }
+      const int64_t k = k0 + threadIdx.x / kL;
+      uint32_t plus = k < v.K ? kBit8 : 0u, minus = plus;
+      if (k < v.K) {
+        const int8_t* g = v.G + k * v.ldg;
+        for (int p = sub; p * 16 < n; p += kL) {
+          const uint4 q = *reinterpret_cast<const uint4*>(g + p * 16);
+          const uint4* room = t.room + 8 * p;
+          room_fits(q.x, room[0], room[1], plus, minus);
+          room_fits(q.y, room[2], room[3], plus, minus);
+          room_fits(q.z, room[4], room[5], plus, minus);
+          room_fits(q.w, room[6], room[7], plus, minus);
+          if ((plus & kBit8) != kBit8 && (minus & kBit8) != kBit8) break;
         }
-        if (kL > 1) {
-#pragma unroll
-          for (int o = kL / 2; o > 0; o >>= 1) {
-            plus &= __shfl_xor_sync(0xffffffffu, plus, o);
-            minus &= __shfl_xor_sync(0xffffffffu, minus, o);
-          }
-        }
-        bool full = false;
-        if (sub == 0 && ((plus & kBit8) == kBit8 || (minus & kBit8) == kBit8)) {
-          const int at = atomicAdd(&s_queued, 1);
-          t.queue[at] = k;
-          full = at >= per_block - 1;
-        }
-        if (!__syncthreads_or(full || last)) continue;
-        cnt = s_queued;
       }
+      if (kL > 1) {
+#pragma unroll
+        for (int o = kL / 2; o > 0; o >>= 1) {
+          plus &= __shfl_xor_sync(0xffffffffu, plus, o);
+          minus &= __shfl_xor_sync(0xffffffffu, minus, o);
+        }
+      }
+      bool full = false;
+      if (sub == 0 && ((plus & kBit8) == kBit8 || (minus & kBit8) == kBit8)) {
+        const int at = atomicAdd(&s_queued, 1);
+        t.queue[at] = first + threadIdx.x / kL;
+        ++fit;
+        full = at >= per_block - 1;
+      }
+      if (!__syncthreads_or(full || last)) continue;
+      const int cnt = s_queued;
       for (int q0 = 0; q0 < cnt; q0 += per_block) {  // a group of lanes each
         const int q = q0 + threadIdx.x / kL;
-        int64_t k = -1;
-        if (pre) {
-          if (q < cnt) k = t.queue[q];
-        } else if (k0 + q < v.K) {
-          k = k0 + q;
+        int64_t kq = -1;
+        if (q < cnt) {
+          const uint32_t at = t.queue[q];
+          kq = ((int64_t)bx + (int64_t)(at / per_block) * v.nb) * per_block + at % per_block;
         }
-        score(k);
+        score(kq);
       }
       if (last) break;
-      if (pre) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_queued = 0;
-        __syncthreads();
-      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_queued = 0;
+      __syncthreads();
     }
+  }
+  if (kVec) {
+    fit = __reduce_add_sync(0xffffffffu, fit);
+    if ((threadIdx.x & 31) == 0 && fit) atomicAdd(&v.fit_now[s], (unsigned long long)fit);
   }
   // block argmin
   __shared__ Best s_best[32];
@@ -632,7 +709,12 @@ __device__ __forceinline__ void apply_body(const AugView& v, int s) {
   }
   __syncthreads();
   best = s_best[0];
-  if (threadIdx.x == 0) v.iters[s] += 1;
+  if (threadIdx.x == 0) {
+    v.iters[s] += 1;
+    v.fit[s] = v.fit_now[s];
+    v.fit_now[s] = 0;
+    v.next[s] = 0;
+  }
   if (best.df >= 0) {  // no improving move: this start is done
     if (threadIdx.x == 0) {
       v.active[s] = 0;
@@ -674,8 +756,10 @@ __device__ __forceinline__ void apply_body(const AugView& v, int s) {
 
 __global__ void __launch_bounds__(kStartThreads) init_kernel(AugView v) { init_body(v, blockIdx.x); }
 
-template <int kL, bool kVec>
-__global__ void score_kernel(AugView v) { score_body<kL, kVec>(v, blockIdx.y, blockIdx.x); }
+template <int kL, bool kVec, bool kQuartic>
+__global__ void __launch_bounds__(kScoreThreads, kQuartic ? 4 : 5) score_kernel(AugView v) {
+  score_body<kL, kVec, kQuartic>(v, blockIdx.y, blockIdx.x);
+}
 
 __global__ void __launch_bounds__(kStartThreads) apply_kernel(AugView v) { apply_body(v, blockIdx.x); }
 
@@ -705,7 +789,8 @@ __global__ void score_batch_kernel(const AugView* __restrict__ items, const int6
   const AugView v = items[i];
   if (*iter >= v.max_iters || v.K == 0) return;
   const int64_t b = blockIdx.x - blk_prefix[i];
-  score_body<kL, kVec>(v, (int)(b / v.nb), (int)(b % v.nb));
+  if (v.w) score_body<kL, kVec, true>(v, (int)(b / v.nb), (int)(b % v.nb));
+  else score_body<kL, kVec, false>(v, (int)(b / v.nb), (int)(b % v.nb));
 }
 
 __global__ void __launch_bounds__(kStartThreads) apply_batch_kernel(const AugView* __restrict__ items, const int64_t* __restrict__ st_prefix,
@@ -743,16 +828,20 @@ using ScoreBatchFn = void (*)(const AugView*, const int64_t*, int, const int64_t
 
 constexpr int kLaneChoices[] = {1, 2, 4, 8, 16, 32};
 
+template <bool kQuartic>
 ScoreFn score_fn(int lanes, bool vec) {
-  if (!vec) return score_kernel<1, false>;
+  if (!vec) return score_kernel<1, false, kQuartic>;
   switch (lanes) {
-    case 1: return score_kernel<1, true>;
-    case 2: return score_kernel<2, true>;
-    case 4: return score_kernel<4, true>;
-    case 8: return score_kernel<8, true>;
-    case 16: return score_kernel<16, true>;
-    default: return score_kernel<32, true>;
+    case 1: return score_kernel<1, true, kQuartic>;
+    case 2: return score_kernel<2, true, kQuartic>;
+    case 4: return score_kernel<4, true, kQuartic>;
+    case 8: return score_kernel<8, true, kQuartic>;
+    case 16: return score_kernel<16, true, kQuartic>;
+    default: return score_kernel<32, true, kQuartic>;
   }
+}
+ScoreFn score_fn(int lanes, bool vec, bool quartic) {
+  return quartic ? score_fn<true>(lanes, vec) : score_fn<false>(lanes, vec);
 }
 
 ScoreBatchFn score_batch_fn(int lanes, bool vec) {
@@ -779,25 +868,30 @@ int score_blocks(int64_t K, int S, int lanes) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(K, per_block), most));
 }
 
-size_t score_smem(int n) {
-  const size_t tables = (size_t)n * (4 * sizeof(long long) + 2 * sizeof(int32_t));
+size_t score_smem(int n, bool quartic) {
+  const size_t tables = (size_t)n * ((quartic ? 4 : 2) * sizeof(long long) + 2 * sizeof(int32_t));
   if (!score_pre(n)) return tables;
   return tables + (n & 1) * sizeof(long long) + (size_t)score_words(n) * 2 * sizeof(uint4) +
-         2 * kScoreThreads * sizeof(int64_t);
+         2 * kScoreThreads * sizeof(uint32_t);
 }
 
-// the shared-memory limit of every variant, where it may take more than the default
-int allow_score_smem(size_t smem, bool batch) {
-  if (smem <= kSmemUnasked) return MAPE_OK;
+// the shared-memory limit of every variant, where it may take more than the
+// default; n: the largest, refused where the quartic term's tables would not
+// fit, with or without one
+int allow_score_smem(size_t smem, int n, bool batch) {
+  const size_t most = std::max(smem, score_smem(n, true));
+  if (most <= kSmemUnasked) return MAPE_OK;
   for (int lanes : kLaneChoices)
-    for (bool vec : {true, false}) {
-      if (!vec && lanes != 1) continue;
-      size_t lim = 0;
-      const void* f = batch ? (const void*)score_batch_fn(lanes, vec) : (const void*)score_fn(lanes, vec);
-      const int rc = allow_max_dynamic_smem(f, &lim);
-      if (rc != MAPE_OK) return rc;
-      if (smem > lim) return MAPE_ERR_SHAPE;
-    }
+    for (bool vec : {true, false})
+      for (bool quartic : {true, false}) {
+        if ((!vec && lanes != 1) || (batch && quartic)) continue;
+        size_t lim = 0;
+        const void* f =
+            batch ? (const void*)score_batch_fn(lanes, vec) : (const void*)score_fn(lanes, vec, quartic);
+        const int rc = allow_max_dynamic_smem(f, &lim);
+        if (rc != MAPE_OK) return rc;
+        if (most > lim) return MAPE_ERR_SHAPE;
+      }
   return MAPE_OK;
 }
 
@@ -833,13 +927,17 @@ AugView make_view(const mape_augment_args* A, long long* R, uint8_t* active, Bes
   v.moves_cap = A->moves_cap;
   v.c = A->c; v.w = A->w; v.l = A->l; v.u = A->u; v.X = A->X; v.fval = A->fval;
   v.moves = A->moves; v.nmoves = nmoves;
+  v.fit = reinterpret_cast<unsigned long long*>(partial + (size_t)A->S * kMaxScoreBlocks);
+  v.fit_now = v.fit + A->S;
+  v.next = v.fit_now + A->S;
   v.R = R; v.active = active; v.partial = partial; v.iters = iters; v.n_active = n_active; v.bad = bad;
   v.max_iters = A->max_iters;
   return v;
 }
 
 // Times one score pass of every lane count on the start's state (the pass
-// writes only the partial minima) and returns the fastest.
+// writes only the partial minima and its counts, which are cleared again) and
+// returns the fastest.
 int tune_lanes(const AugView& base, size_t smem, cudaStream_t st, mape_augment_tune_info* out) {
   cudaEvent_t e0, e1;
   MAPE_CUDA_TRY(cudaEventCreate(&e0));
@@ -852,8 +950,9 @@ int tune_lanes(const AugView& base, size_t smem, cudaStream_t st, mape_augment_t
     v.nb = score_blocks(v.K, v.S, lanes);
     float ms = 0.f;
     for (int rep = 0; rep < 2; ++rep) {  // the first launch loads the kernel
+      MAPE_CUDA_TRY(cudaMemsetAsync(base.next, 0, sizeof(unsigned long long) * base.S, st));
       MAPE_CUDA_TRY(cudaEventRecord(e0, st));
-      launch(score_fn(lanes, true), dim3((unsigned)v.nb, (unsigned)v.S), kScoreThreads, smem, st, v);
+      launch(score_fn(lanes, true, v.w != nullptr), dim3((unsigned)v.nb, (unsigned)v.S), kScoreThreads, smem, st, v);
       MAPE_CUDA_TRY(cudaEventRecord(e1, st));
       MAPE_CUDA_TRY(cudaEventSynchronize(e1));
       MAPE_CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
@@ -868,6 +967,7 @@ int tune_lanes(const AugView& base, size_t smem, cudaStream_t st, mape_augment_t
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  MAPE_CUDA_TRY(cudaMemsetAsync(base.fit_now, 0, 2 * sizeof(unsigned long long) * base.S, st));  // and next
   out->candidates = nc;
   return MAPE_OK;
 }
@@ -936,7 +1036,7 @@ AugCarve carve(const mape_augment_args* A) {
   AugCarve c{};
   c.R = cv.take<long long>((size_t)S * n);
   c.active = cv.take<uint8_t>((size_t)S);
-  c.partial = cv.take<Best>((size_t)S * kMaxScoreBlocks);
+  c.partial = cv.take<Best>((size_t)S * kMaxPartials);
   c.iters = cv.take<int32_t>((size_t)S);
   c.n_active = cv.take<unsigned int>(1);
   c.bad = cv.take<int32_t>(1);
@@ -1055,7 +1155,7 @@ extern "C" size_t mape_augment_workspace_bytes(int32_t n, int32_t S, int64_t K) 
   Sizer s;
   s.take<long long>((size_t)S * n);          // R
   s.take<uint8_t>((size_t)S);                // active
-  s.take<Best>((size_t)S * kMaxScoreBlocks); // partial minima
+  s.take<Best>((size_t)S * kMaxPartials);    // partial minima
   s.take<int32_t>((size_t)S);                // per-start iteration counts
   s.take<unsigned int>(1);                   // active count
   s.take<int32_t>(1);                        // bad-start flag
@@ -1093,12 +1193,12 @@ extern "C" int mape_augment_run(const mape_augment_args* A, int64_t* iters_out, 
     *iters_out = 1;
     return MAPE_OK;
   }
-  const size_t smem = score_smem(n);
-  if ((rc = allow_score_smem(smem, false)) != MAPE_OK) return rc;
+  const size_t smem = score_smem(n, A->w != nullptr);
+  if ((rc = allow_score_smem(smem, n, false)) != MAPE_OK) return rc;
   int lanes = 1;
   if ((rc = pick_lanes(A, v, vec, smem, st, &lanes)) != MAPE_OK) return rc;
   v.nb = score_blocks(K, S, lanes);
-  const ScoreFn score = score_fn(lanes, vec);
+  const ScoreFn score = score_fn(lanes, vec, v.w != nullptr);
   int64_t done_iters = 0;
   const int64_t chunk = 8;
   while (done_iters < A->max_iters) {
@@ -1163,13 +1263,15 @@ extern "C" int mape_augment_run_batch(const mape_augment_args* items, int32_t co
   bool vec = true;
   int lanes = items[0].score_lanes, big = 0;
   size_t smem = 0;
+  int max_n = 0;
   for (int i = 0; i < count; ++i) {
     const mape_augment_args* A = &items[i];
     if (A->S == 0) continue;
     if (A->K > 0 && !rows_vectorisable(A)) vec = false;
     if (A->score_lanes != lanes) lanes = 0;
     if (A->K * A->n > items[big].K * items[big].n) big = i;
-    smem = std::max(smem, score_smem(A->n));
+    smem = std::max(smem, score_smem(A->n, A->w != nullptr));
+    max_n = std::max(max_n, A->n);
   }
   std::vector<AugView> views((size_t)count);
   std::vector<AugCarve> carves((size_t)count);
@@ -1222,7 +1324,7 @@ extern "C" int mape_augment_run_batch(const mape_augment_args* items, int32_t co
       for (int i = 0; i < count; ++i) done(i, iters_out[i], done_ctx);
     return MAPE_OK;
   }
-  if ((rc = allow_score_smem(smem, true)) != MAPE_OK) return rc;
+  if ((rc = allow_score_smem(smem, max_n, true)) != MAPE_OK) return rc;
   if (!vec) {
     lanes = 1;
   } else if (lanes == 0) {
