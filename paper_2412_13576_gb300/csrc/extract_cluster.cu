@@ -32,6 +32,11 @@
 // the same SM; the resident kernel (116 KB, 512 columns) never shares an SM with
 // them.
 //
+// The tensor-memory loads and their waits are for a converged warp, which the
+// code between them does not leave (lane 0 arrives on a barrier, lanes write
+// their debug outputs): without a __syncwarp before each, halves of a warp
+// took a chunk's gradient before it was there.  The four cost 1% of a step.
+//
 // Accumulation order: K ascends in steps of 16, hi before lo, into one FP32
 // accumulator per (start, row), the order of the step-by-step kernels of
 // extract_stream.cu; the gradient's sums are integers.  Both give the same
@@ -540,6 +545,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
             const int i0 = row0 + rb + ch * 16;
             uint32_t v[16];
             if (do_fwd) {
+              __syncwarp();
               tmem_ld16(tmem + lane_base + ch * 16, v);
               tc_wait_ld();
               uint32_t w[8];
@@ -554,6 +560,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
               *reinterpret_cast<uint4*>(Sp + off16(r, (i0 & 31) + 8)) = make_uint4(w[4], w[5], w[6], w[7]);
             }
             if (coll) {
+              __syncwarp();
               tmem_ld16(tmem + lane_base + kColD2 + ch * 16, v);
               tc_wait_ld();
               uint32_t pk[4] = {0, 0, 0, 0};
@@ -702,6 +709,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
         auto chunk = [&](int ch) {
           const int j0 = col0 + cb + ch * 8;
           uint32_t gv[8];
+          __syncwarp();
           tmem_ld8(tmem + lane_base + ch * 8, gv);
           const uint32_t e = ec + (uint32_t)(cb / 8 + ch), st = e % kEStages;
           if (!wait_or_abort(efull0 + 8 * st, (e / kEStages) & 1u)) ok = false;
@@ -724,6 +732,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
             const float e = zc[k] - rz[k];
             g[k] = fmaf(-2.f, e, sgn_sat(e));
           }
+          __syncwarp();
           tc_wait_ld();
 #pragma unroll
           for (int k = 0; k < 8; ++k) g[k] = fmaf(p.lambda1, g[k], __uint_as_float(gv[k]));
