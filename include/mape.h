@@ -93,9 +93,11 @@ extern "C" {
  *   streamed: tiles of 128 starts with B and the state streamed through
  *             shared memory by bulk copies; any n, d <= 4096.  An
  *             identity-topped B runs in one launch for all T steps, a cluster
- *             of thread blocks per tile; a general B (and every B while
- *             mape_launch_timing is on) in three kernels per step (forward +
- *             map, collect, gradient + Adam).  Both give the same bits.
+ *             of thread blocks per tile (but for some numbers of tiles of n >
+ *             640 that fill the last wave too little); a general B (and in
+ *             mape_extract every B while mape_launch_timing is on) in three
+ *             kernels per step (forward + map, collect, gradient + Adam).
+ *             Both give the same bits.
  * The resident kernel is chosen when it fits; OR-ing MAPE_PREC_STREAMED into
  * the precision forces the streamed one. */
 #define MAPE_PREC_STREAMED 0x100
@@ -856,8 +858,9 @@ void mape_server_destroy(mape_server_h s);
  * of launches since timing was switched on (or last read: reading clears the
  * pending pairs, not the sums).  mape_launch_timing(enable) switches it and
  * clears everything.  The events add a little time around each launch, so
- * time a region either with or without it.  While it is on, streamed calls run
- * step by step for every B, since these kinds are launches of one step. */
+ * time a region either with or without it.  While it is on, the streamed calls
+ * of mape_extract run step by step for every B, since these kinds are launches of
+ * one step; mape_extract_batch runs as ever and reports none of them. */
 #define MAPE_TIMED_STREAM_FWD     0   /* streamed forward + map kernel       */
 #define MAPE_TIMED_STREAM_COLLECT 1   /* streamed collection kernel          */
 #define MAPE_TIMED_STREAM_GRAD    2   /* streamed gradient + Adam kernel     */

@@ -1155,17 +1155,53 @@ void cl_carve(Carve& cv, const ClShape& sh, int32_t precision, ClCarved* c) {
 
 namespace mape_detail {
 
-// Blocks per cluster of a call.  Two blocks fit an SM, so 8-block clusters of
-// 38 tiles fill the chip: up to there a step is bound by the latency of its
-// phases, which 8 slices shorten (n = 1000, P = 4096: 29.1 us a step against
-// 30.0 with 4 blocks and 48 with 2; P = 1024: 21.8, 29, 46).  Beyond, tiles wait
-// for an SM anyway, and 4 slices read the shared operands half as often
-// (n = 1000, P = 16384: 72 us against 97; n = 2000, P = 65536 in BF16: 586
-// against 667, in FP8 469 against 467).
-static int cl_blocks(int64_t tiles) { return tiles * kMaxC <= 2 * kSms ? kMaxC : 4; }
-
-// ... of a call in a batch, whose tiles run beside many others
-static int cl_blocks_batch(int d32) { return d32 >= 512 ? 8 : d32 >= 256 ? 4 : 2; }
+// Blocks per cluster of a call, and their shared memory, by the tiles that run
+// together (of the call, or of its whole batch).  More blocks per tile
+// shorten a step (its latency is a part that stays and one that is shared), as
+// long as all tiles run at once; clusters stay within a GPC, so that 15 of 8 blocks,
+// 36 of 4 and 76 of 2 run with an SM per block, 36 of 8, 74 of 4 and 152 of 2
+// with two blocks to an SM.  One tile more is a second wave: n = 487, 20 steps,
+// us: 36 tiles 0.50 ms with 8 and 4 blocks, 37 tiles 0.78 and 0.59; 73 tiles 0.65
+// with 4, 76 tiles 0.99, 0.70 with 2.  Where the lines lie otherwise:
+//  16 .. 36 tiles: 4 blocks with an SM each take 0.93 to 0.98 of the time of 8 with
+//    two to an SM for n = 20 to 60, 1.02 to 1.09 for n = 100 to 2000;
+//  .. 74 tiles: 2 blocks an SM each take 0.94 of the time of 4 for n = 20, 1.05 to
+//    1.2 from n = 125 on;
+//  77 .. 152 tiles, d > 1024: two waves of 4 blocks 4.6 ms against 5.0 with 2 (n =
+//    2000, 128 tiles), 2.18 and 2.13 for n = 1000;
+//  beyond: tiles wait for an SM anyway, and for small n the fewer blocks share a
+//    tile the less is spent on barriers (512 tiles of n = 50, 200, 487, 700: 0.81,
+//    1.33, 3.99, 5.96 ms with 1 block, 1.60, 2.17, 3.93, 5.54 with 4).
+// False: the step-by-step kernels, where waves of 4 blocks leave the chip too
+// empty for the gain of a step (1.2 at n = 2000 with full waves) to make up for
+// it.  Collecting every step, BF16: n = 2000, 77, 101, 153 and 178 tiles 3.64, 4.20,
+// 6.27 and 6.49 ms against 3.25, 3.95, 5.51 and 6.34, but 128 tiles 4.57 and 4.69; n =
+// 1000, 153 tiles 3.02 and 2.79; n = 550 1.61 and 1.73.  Every second step: 75
+// tiles 3.32 and 2.94, 101 3.76 and 3.67, 121 3.99 and 4.21.  More rows below the
+// identity than coordinates (n = 1300, d = 120), 223 tiles: 2.99 and 2.63, FP8 2.95
+// and 2.73.  FP8 is faster in clusters at the other sizes (n = 2000: 3.36, 3.77, 5.57
+// against 3.44, 4.10, 5.70).
+struct ClChoice {
+  int C, dyn;
+};
+static bool cl_choose(const mape_extract_args* a, int64_t tiles, ClChoice* c) {
+  const int n = a->n, d = a->d;
+  if (tiles <= 15) *c = {8, kDynSmemOne};
+  else if (tiles <= 36) *c = n <= 64 ? ClChoice{4, kDynSmemOne} : ClChoice{8, kDynSmem};
+  else if (tiles <= 74 && n > 64) *c = {4, kDynSmem};
+  else if (tiles <= 76 && d <= 1024) *c = {2, kDynSmemOne};
+  else if (tiles <= 152 && d <= 1024) *c = {2, kDynSmem};
+  else if (n <= 320) *c = {1, kDynSmem};
+  else {
+    *c = {4, kDynSmem};
+    if (n <= 640) return true;
+    if (n - d > d) return false;
+    const bool often = a->precision == MAPE_PREC_BF16 && a->period == 1;
+    if (a->precision == MAPE_PREC_FP8 || (!often && n <= 800)) return true;
+    return 100 * tiles >= (often ? 84 : 76) * 74 * ceil_div(tiles, 74);
+  }
+  return true;
+}
 
 size_t extract_cluster_workspace(int32_t n, int32_t d, int32_t P, int32_t precision) {
   if (d >= n) return 0;
@@ -1174,11 +1210,11 @@ size_t extract_cluster_workspace(int32_t n, int32_t d, int32_t P, int32_t precis
   return s.bytes();
 }
 
-static void cl_params(const ClCarved& c, const mape_extract_args* a, int C, ClParams& p) {
+static void cl_params(const ClCarved& c, const mape_extract_args* a, ClChoice choice, ClParams& p) {
   const ClShape& sh = c.sh;
   p = ClParams{};
   p.n = a->n; p.d = a->d; p.P = a->P; p.R = sh.R; p.d32 = sh.d32; p.R32 = sh.R32; p.d64 = sh.d64;
-  p.tiles = sh.tiles; p.C = C; p.dyn = kDynSmem; p.ldc = a->ldc; p.mapoff = sh.mapoff; p.lds = sh.lds;
+  p.tiles = sh.tiles; p.C = choice.C; p.dyn = choice.dyn; p.ldc = a->ldc; p.mapoff = sh.mapoff; p.lds = sh.lds;
   p.Bf = c.Bf; p.Bf8 = c.Bf8; p.Bg = c.Bg; p.span = a->span; p.Zt = c.Zt; p.Mt = c.Mt; p.Vt = c.Vt;
   p.Zh = c.Zh; p.S = c.S; p.stage = c.stage; p.zkey = c.zkey; p.acc = c.acc;
   p.oob = c.oob; p.idw = c.idw; p.first = c.first; p.bias = c.bias;
@@ -1246,11 +1282,13 @@ static int launch_clusters(void (*kernel)(KArgs...), int64_t clusters, int C, in
   return MAPE_OK;
 }
 
-// One call.  *general = true (and nothing done) when B has no identity top.
+// One call.  *general = true (and nothing done) when B has no identity top, or
+// the step-by-step kernels are faster.
 int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general) {
   *general = false;
   if (a->T > kBiasSteps) return MAPE_ERR_SHAPE;
-  if (a->d >= a->n) { *general = true; return MAPE_OK; }
+  ClChoice choice;
+  if (a->d >= a->n || !cl_choose(a, ceil_div(a->P, kTM), &choice)) { *general = true; return MAPE_OK; }
   Carver cv(a->workspace, a->workspace_bytes);
   ClCarved c;
   cl_carve(cv, cl_shape(a->n, a->d, a->P), a->precision, &c);
@@ -1260,8 +1298,7 @@ int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general) 
   if (rc != MAPE_OK) return rc;
   if (!ids[0]) { *general = true; return MAPE_OK; }
   ClParams p;
-  cl_params(c, a, cl_blocks(c.sh.tiles), p);
-  if ((int64_t)p.tiles * p.C <= kSms) p.dyn = kDynSmemOne;
+  cl_params(c, a, choice, p);
   if ((rc = cl_pack(p, a, c.hflags + 1, st)) != MAPE_OK) return rc;
   int32_t h_bad = 0;
   MAPE_CUDA_TRY(cudaMemcpyAsync(&h_bad, c.hflags + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1328,7 +1365,14 @@ int extract_cluster_batch_prepare(const mape_extract_args* const* items, int cou
     Carver cv(a->workspace, a->workspace_bytes);
     cl_carve(cv, cl_shape(a->n, a->d, a->P), a->precision, &carved[i]);
     if (!cv.ok) return MAPE_ERR_CAPACITY;
-    cl_params(carved[i], a, cl_blocks_batch(carved[i].sh.d32), plan->params[i]);
+    // by the tiles of the whole batch: 0.75 to 0.95 of the time of a rule by d
+    // alone (8 blocks from 512 coordinates on, 4 from 256, else 2), which for 8
+    // calls of n = 1000 and P = 16384 was slower than the step-by-step kernels
+    // (22.3 ms against 20.9; 18.3 now)
+    ClChoice choice;
+    cl_choose(a, tiles, &choice);
+    choice.dyn = kDynSmem;
+    cl_params(carved[i], a, choice, plan->params[i]);
     if ((rc = cl_pack(plan->params[i], a, carved[i].hflags + 1, st)) != MAPE_OK) return rc;
   }
   std::vector<int32_t> bad((size_t)count, 0);

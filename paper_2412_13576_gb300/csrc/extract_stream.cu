@@ -1426,9 +1426,10 @@ int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, i
 
 // The default implementation: one launch of tile clusters for an
 // identity-topped B (extract_cluster.cu, 2 to 3.5 times faster a step up to
-// P = 4096, 1.15 to 1.27 times at P = 65536), the step-by-step kernels at
-// their widest blocks for a general B, for the sparse forward, and while
-// launch timing is on, whose kinds are those kernels.  The same bits either way.
+// P = 4096, 1.1 to 2 times at P = 65536) except at the sizes that cl_choose
+// there names, the step-by-step kernels at their widest blocks for those, for a
+// general B, for the sparse forward, and while launch timing is on, whose kinds
+// are those kernels.  The same bits either way.
 int extract_stream(const mape_extract_args* a, cudaStream_t st, int fwd_mode) {
   if (fwd_mode == kFwdDense && !launch_timing_on()) {
     bool general = false;
