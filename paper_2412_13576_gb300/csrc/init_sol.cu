@@ -56,9 +56,16 @@ struct InitParams {
   float2* rows;      // group g of 32 rows at g * 32 * cap_r: entry e of row i at e * 32 + i % 32
   float2* cols;      // the same for columns, cap_c entries
   int32_t* width;    // longest list per group of rows, then per group of columns
-  int32_t* dense;    // 1: some list is longer than its capacity
   int cap_r, cap_c;
 };
+
+// by every lane of a warp: some list of A is longer than its capacity
+__device__ __forceinline__ bool lists_overflow(const InitParams& p) {
+  const int gr = (p.m + 31) / 32, groups = gr + (p.n + 31) / 32;
+  bool over = false;
+  for (int i = threadIdx.x & 31; i < groups; i += 32) over |= p.width[i] > (i < gr ? p.cap_r : p.cap_c);
+  return __any_sync(0xffffffffu, over) != 0;
+}
 
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
@@ -66,9 +73,7 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-__global__ void __launch_bounds__(32 * kWarps) init_sol_kernel(InitParams p) {
-  extern __shared__ __align__(16) float sm[];
-  if (*p.dense == 0) return;
+__device__ __forceinline__ void dense_steps(const InitParams& p, float* sm) {
   const int n = p.n, m = p.m;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* sAf = sm;
@@ -163,47 +168,69 @@ __global__ void __launch_bounds__(32 * kWarps) init_sol_kernel(InitParams p) {
   for (int j = lane; j < n; j += 32) X[j] = xs[j];
 }
 
-// Lists of the nonzeros of A.  Row part (a warp per row): the row's nonzeros in
-// column order; column part (a warp per 32 columns): in row order.
-__global__ void init_lists_kernel(const int32_t* __restrict__ A, InitParams p) {
-  const int lane = threadIdx.x & 31;
-  const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  const int n = p.n, m = p.m;
-  if (w < m) {
-    float2* out = p.rows + (size_t)(w >> 5) * 32 * p.cap_r + (w & 31);
+// What the steps read of A, in one launch (small calls are bound by their
+// launches: a kernel each and a cleared flag cost 256 starts of a 20 x 5 matrix
+// 6% of 175 us).  The first blocks: the nonzeros of 32 rows, a warp per row, in
+// column order.  The next: those of 32 x 32 columns, a warp per 32 columns, in
+// row order.  The rest: A as FP32 in both orientations.
+constexpr int kSetupThreads = 1024;
+
+__global__ void __launch_bounds__(kSetupThreads) init_setup_kernel(const int32_t* __restrict__ A, InitParams p,
+                                                                   float* __restrict__ Af, float* __restrict__ At) {
+  const int n = p.n, m = p.m, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gr = (m + 31) / 32, gc = (n + 31) / 32;
+  int b = blockIdx.x;
+  if (b < gr) {
+    __shared__ int s_most[kSetupThreads / 32];
+    const int w = b * 32 + warp;
     int at = 0;
-    for (int j0 = 0; j0 < n; j0 += 32) {
-      const int j = j0 + lane;
-      const int v = j < n ? A[(int64_t)w * n + j] : 0;
-      const unsigned bal = __ballot_sync(0xffffffffu, v != 0);
-      const int e = at + __popc(bal & ((1u << lane) - 1));
-      if (v != 0 && e < p.cap_r) out[(size_t)e * 32] = make_float2((float)v, __int_as_float(j));
-      at += __popc(bal);
+    if (w < m) {
+      float2* out = p.rows + (size_t)b * 32 * p.cap_r + warp;
+      for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane;
+        const int v = j < n ? A[(int64_t)w * n + j] : 0;
+        const unsigned bal = __ballot_sync(0xffffffffu, v != 0);
+        const int e = at + __popc(bal & ((1u << lane) - 1));
+        if (v != 0 && e < p.cap_r) out[(size_t)e * 32] = make_float2((float)v, __int_as_float(j));
+        at += __popc(bal);
+      }
+      for (int e = at + lane; e < p.cap_r; e += 32) out[(size_t)e * 32] = make_float2(0.f, __int_as_float(0));
     }
-    if (lane == 0) {
-      if (at > p.cap_r) atomicOr(p.dense, 1);
-      atomicMax(&p.width[w >> 5], at);
+    if (lane == 0) s_most[warp] = at;
+    __syncthreads();
+    if (warp == 0) {
+      const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)s_most[lane]);
+      if (lane == 0) p.width[b] = most;
     }
-    for (int e = at + lane; e < p.cap_r; e += 32) out[(size_t)e * 32] = make_float2(0.f, __int_as_float(0));
     return;
   }
-  const int g = w - m;  // group of columns
-  if (g >= (n + 31) / 32) return;
-  const int j = g * 32 + lane;
-  float2* out = p.cols + (size_t)g * 32 * p.cap_c + lane;
-  int at = 0;
+  b -= gr;
+  if (b < (gc + 31) / 32) {
+    const int g = b * 32 + warp;  // group of columns
+    if (g >= gc) return;
+    const int j = g * 32 + lane;
+    float2* out = p.cols + (size_t)g * 32 * p.cap_c + lane;
+    int at = 0;
 #pragma unroll 4
-  for (int i = 0; i < m; ++i) {
-    const int v = j < n ? A[(int64_t)i * n + j] : 0;
-    if (v != 0) {
-      if (at < p.cap_c) out[(size_t)at * 32] = make_float2((float)v, __int_as_float(i));
-      ++at;
+    for (int i = 0; i < m; ++i) {
+      const int v = j < n ? A[(int64_t)i * n + j] : 0;
+      if (v != 0) {
+        if (at < p.cap_c) out[(size_t)at * 32] = make_float2((float)v, __int_as_float(i));
+        ++at;
+      }
     }
+    const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)at);
+    if (lane == 0) p.width[gr + g] = most;
+    for (int e = at; e < most && e < p.cap_c; ++e) out[(size_t)e * 32] = make_float2(0.f, __int_as_float(0));
+    return;
   }
-  if (at > p.cap_c) atomicOr(p.dense, 1);
-  const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)at);
-  if (lane == 0) p.width[(m + 31) / 32 + g] = most;
-  for (int e = at; e < most && e < p.cap_c; ++e) out[(size_t)e * 32] = make_float2(0.f, __int_as_float(0));
+  b -= (gc + 31) / 32;
+  const int64_t e = b * (int64_t)kSetupThreads + threadIdx.x;
+  if (e >= (int64_t)m * n) return;
+  const int i = (int)(e / n), j = (int)(e % n);
+  const float v = (float)A[e];
+  Af[e] = v;
+  At[(int64_t)j * m + i] = v;
 }
 
 // sum of value x vec[index] over a list of `width` entries, from acc, in order
@@ -231,9 +258,7 @@ constexpr int kListThreads = 128;  // per start
 // kNT > 0: n <= 128 kNT, the moments and bounds of a thread's coordinates in
 // registers for the whole call; 0: any n, in global memory.
 template <int kNT>
-__global__ void __launch_bounds__(kListThreads) init_sol_lists_kernel(InitParams p) {
-  extern __shared__ __align__(16) float sm[];
-  if (*p.dense != 0) return;
+__device__ __forceinline__ void list_steps(const InitParams& p, float* sm) {
   const int n = p.n, m = p.m;
   const int tid = threadIdx.x, lane = tid & 31;
   float* xs = sm;
@@ -371,18 +396,30 @@ __global__ void __launch_bounds__(kListThreads) init_sol_lists_kernel(InitParams
   for (int j = tid; j < n; j += kListThreads) X[j] = xs[j];
 }
 
+__global__ void __launch_bounds__(32 * kWarps) init_sol_kernel(InitParams p) {
+  extern __shared__ __align__(16) float sm[];
+  if (lists_overflow(p)) dense_steps(p, sm);
+}
+// the registers that the moments leave: 12, 10, 8 and 9 blocks an SM
+template <int kNT>
+__global__ void __launch_bounds__(kListThreads, kNT == 1 ? 12 : kNT == 2 ? 10 : kNT == 4 ? 8 : 9)
+init_sol_lists_kernel(InitParams p) {
+  extern __shared__ __align__(16) float sm[];
+  if (!lists_overflow(p)) list_steps<kNT>(p, sm);
+}
+// the two in one launch, of a block per start: for the smallest A (a launch for
+// nothing is 3 us; with the 9.5 KB of 64 x 16 entries the dense steps take 475 us
+// here, 440 in their own kernel)
+static_assert(kListThreads == 32 * kWarps);
+constexpr size_t kBothSmem = 4 * 1024;
+__global__ void __launch_bounds__(kListThreads) init_sol_both_kernel(InitParams p) {
+  extern __shared__ __align__(16) float sm[];
+  if (!lists_overflow(p)) list_steps<1>(p, sm);
+  else if (blockIdx.x < (unsigned)((p.P + kWarps - 1) / kWarps)) dense_steps(p, sm);
+}
+
 int list_cap(int x) { return x / 2 + 1; }
 size_t list_entries(int lists, int cap) { return (size_t)((lists + 31) / 32) * 32 * cap; }
-
-__global__ void init_operands_kernel(const int32_t* __restrict__ A, int m, int n, float* __restrict__ Af,
-                                     float* __restrict__ At) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= (int64_t)m * n) return;
-  const int i = (int)(e / n), j = (int)(e % n);
-  const float v = (float)A[e];
-  Af[e] = v;
-  At[(int64_t)j * m + i] = v;
-}
 
 }  // namespace
 
@@ -394,7 +431,7 @@ extern "C" size_t mape_initial_solutions_workspace_bytes(int32_t n, int32_t m, i
   s.take<float2>((size_t)(T > 0 ? T : 1));
   s.take<float2>(list_entries(m, list_cap(n)));
   s.take<float2>(list_entries(n, list_cap(m)));
-  s.take<int32_t>((size_t)(m + 31) / 32 + (n + 31) / 32 + 1);
+  s.take<int32_t>((size_t)(m + 31) / 32 + (n + 31) / 32);
   return s.bytes();
 }
 
@@ -416,8 +453,8 @@ extern "C" int mape_initial_solutions(const mape_init_args* a, void* stream) {
   float2* bias = cv.take<float2>((size_t)a->T);
   float2* rows = cv.take<float2>(list_entries(m, list_cap(n)));
   float2* cols = cv.take<float2>(list_entries(n, list_cap(m)));
-  const size_t groups = (size_t)(m + 31) / 32 + (n + 31) / 32;
-  int32_t* width = cv.take<int32_t>(groups + 1);  // and the dense flag
+  const int gr = (m + 31) / 32, gc = (n + 31) / 32;
+  int32_t* width = cv.take<int32_t>((size_t)gr + gc);
   if (!cv.ok) return MAPE_ERR_CAPACITY;
   std::vector<float2> bc((size_t)a->T);
   for (int s = 0; s < a->T; ++s) {
@@ -426,7 +463,6 @@ extern "C" int mape_initial_solutions(const mape_init_args* a, void* stream) {
     bc[s] = make_float2((float)((double)a->lr / bc1), (float)(1.0 / std::sqrt(bc2)));
   }
   MAPE_CUDA_TRY(cudaMemcpyAsync(bias, bc.data(), sizeof(float2) * bc.size(), cudaMemcpyHostToDevice, st));
-  launch(init_operands_kernel, (unsigned)ceil_div((int64_t)m * n, 256), 256, 0, st, a->A, m, n, Af, At);
   InitParams p{};
   p.n = n; p.m = m; p.P = P; p.t0 = a->t0; p.T = a->T; p.period = a->period;
   p.Af = Af; p.At = At; p.b = a->b; p.l = a->l; p.u = a->u; p.X = a->X; p.M = a->M; p.V = a->V; p.bias = bias;
@@ -435,10 +471,10 @@ extern "C" int mape_initial_solutions(const mape_init_args* a, void* stream) {
   p.omb1 = (float)(1.0 - a->beta1); p.omb2 = (float)(1.0 - a->beta2);
   p.sol = a->sol; p.lds = a->lds; p.cap = a->sol_cap; p.count = a->sol_count; p.flags = a->flags;
   p.dbg_f = a->dbg_f; p.dbg_grad = a->dbg_grad;
-  p.rows = rows; p.cols = cols; p.width = width; p.dense = width + groups;
+  p.rows = rows; p.cols = cols; p.width = width;
   p.cap_r = list_cap(n); p.cap_c = list_cap(m);
-  MAPE_CUDA_TRY(cudaMemsetAsync(width, 0, sizeof(int32_t) * (groups + 1), st));
-  launch(init_lists_kernel, (unsigned)ceil_div(((int64_t)m + (n + 31) / 32) * 32, 256), 256, 0, st, a->A, p);
+  launch(init_setup_kernel, (unsigned)(gr + ceil_div(gc, 32) + ceil_div((int64_t)m * n, kSetupThreads)), kSetupThreads, 0,
+         st, a->A, p, Af, At);
   const size_t per_warp = (size_t)kWarps * (n + m) * sizeof(float);
   const size_t with_a = 2 * (size_t)m * n * sizeof(float) + per_warp;
   p.a_smem = with_a <= kSmemLimit ? 1 : 0;
@@ -450,10 +486,15 @@ extern "C" int mape_initial_solutions(const mape_init_args* a, void* stream) {
     if (rc != MAPE_OK) return rc;
     if ((size_t)smem > lim) return MAPE_ERR_SHAPE;
   }
+  const size_t lsm = (size_t)(n + m) * sizeof(float);
+  if (n <= 128 && smem <= kBothSmem) {  // holds the lists' lsm, too
+    launch(init_sol_both_kernel, (unsigned)P, kListThreads, smem, st, p);
+    MAPE_LAUNCH_CHECK();
+    return MAPE_OK;
+  }
   launch(init_sol_kernel, (unsigned)ceil_div(P, kWarps), 32 * kWarps, smem, st, p);
   auto lists = n <= 128 ? init_sol_lists_kernel<1> : n <= 256 ? init_sol_lists_kernel<2>
              : n <= 512 ? init_sol_lists_kernel<4> : init_sol_lists_kernel<0>;
-  const size_t lsm = (size_t)(n + m) * sizeof(float);
   if (lsm > kSmemUnasked) {
     size_t lim = 0;
     const int rc = allow_max_dynamic_smem((const void*)lists, &lim);
