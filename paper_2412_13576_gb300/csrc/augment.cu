@@ -149,6 +149,12 @@ __device__ __forceinline__ void coeffs_rows(const int32_t* __restrict__ qr, cons
 // words a lane, where the rows-per-warp kernel above loaded two bytes a product
 // and was bound by their bank conflicts: 1.40 ms for 225 000 directions of 2000
 // entries, 10 014 entries of Q and the quartic term, 0.76 here.
+// A tile has its transposition, barriers and sums to pay for, which a short Q
+// does not give back; measured from n = 16 to 2000 with 300 000 rows, tiles
+// against rows per warp: n = 50, 300 entries 142 and 92 us, 1250 entries 193 and
+// 198; n = 200, 1200 entries 195 and 184, 2400 266 and 300; n = 400, 400 entries
+// 168 and 111, 1200 209 and 214; n = 1000, 1000 entries 208 and 236.
+constexpr int64_t kCoefTileWork = 1850;  // entries and twice the coordinates
 constexpr int kCoefThreads = 512, kCoefChunk = 1024;
 static_assert(kCoefChunk / (kCoefThreads / kTileLanes) == 16);
 
@@ -234,16 +240,17 @@ coeffs_tile_kernel(const int32_t* __restrict__ qr, const int32_t* __restrict__ q
   }
 }
 
-// rows at any pitch and address, byte by byte; dynamic shared memory: kCoefWarps x kCoefRows rows of ldg bytes
+// Directions that are not 16-byte aligned (byte by byte), and aligned ones with a
+// short Q; dynamic shared memory: kCoefWarps x kCoefRows rows of ldg bytes
 __global__ void coeffs_kernel(const int32_t* __restrict__ qr, const int32_t* __restrict__ qc,
                               const int32_t* __restrict__ qv, int nnz, const int32_t* __restrict__ w, int n,
-                              const int8_t* __restrict__ G, int64_t K, int ldg, int64_t* __restrict__ a,
+                              const int8_t* __restrict__ G, int64_t K, int ldg, int vec, int64_t* __restrict__ a,
                               int64_t* __restrict__ q4) {
   extern __shared__ __align__(16) int8_t s_rows[];
   const int wid = threadIdx.x >> 5;
   const int64_t k0 = ((int64_t)blockIdx.x * kCoefWarps + wid) * kCoefRows;
   if (k0 >= K) return;  // warp-uniform
-  coeffs_rows(qr, qc, qv, nnz, w, n, G, k0, (int)(K - k0 < kCoefRows ? K - k0 : kCoefRows), ldg, 0,
+  coeffs_rows(qr, qc, qv, nnz, w, n, G, k0, (int)(K - k0 < kCoefRows ? K - k0 : kCoefRows), ldg, vec,
               s_rows + (size_t)wid * kCoefRows * ldg, a, q4);
 }
 
@@ -1073,7 +1080,8 @@ extern "C" int mape_direction_coeffs(const int32_t* q_row, const int32_t* q_col,
     return MAPE_ERR_INVALID_ARG;
   if (K == 0) return MAPE_OK;
   if (ldg > kCoefMaxRow) return MAPE_ERR_SHAPE;
-  if (ldg % 16 == 0 && (reinterpret_cast<uintptr_t>(G) & 15) == 0) {
+  const bool vec = ldg % 16 == 0 && (reinterpret_cast<uintptr_t>(G) & 15) == 0;
+  if (vec && nnz + 2ll * n >= kCoefTileWork) {
     const size_t tile = tile_bytes(n) + sizeof(int4) * kCoefChunk;
     if (tile > kSmemUnasked) {
       size_t lim = 0;
@@ -1094,7 +1102,7 @@ extern "C" int mape_direction_coeffs(const int32_t* q_row, const int32_t* q_col,
     if (smem > lim) return MAPE_ERR_SHAPE;
   }
   mape_detail::launch(coeffs_kernel, (unsigned)ceil_div(K, (int64_t)kCoefWarps * kCoefRows), 32 * kCoefWarps, smem,
-                      as_stream(stream), q_row, q_col, q_val, nnz, w, n, G, K, ldg, a, q4);
+                      as_stream(stream), q_row, q_col, q_val, nnz, w, n, G, K, ldg, vec ? 1 : 0, a, q4);
   MAPE_LAUNCH_CHECK();
   return MAPE_OK;
 }
