@@ -84,7 +84,7 @@ __global__ void kernel_test_kernel(const int32_t* __restrict__ A, int m, int n, 
 // warp per row of A.  When every row of A has sum |a| <= kTileSum they are
 // packed for the tile kernel (pack[q] = tile_at(column) | value << kTileShift,
 // start[r] = the sum's start, see there); else *big is set and they are col, val.
-// A row of a small sum is filled up with zero entries to a multiple of four
+// While every row does, each is filled up with zero entries to a multiple of four
 // (*big is set where that would take more than the n entries there is room for).
 constexpr int kTileSum = 255, kTileShift = 17;
 
@@ -105,10 +105,8 @@ __global__ void csr_count_kernel(const int32_t* __restrict__ A, int m, int n, ui
     sum += __shfl_xor_sync(0xffffffffu, sum, off);
   }
   if (lane == 0) {
-    const uint32_t c4 = (c + 3) & ~3u;
-    const bool fits = sum <= kTileSum && c4 <= (uint32_t)n;
-    rowcnt[r] = fits ? c4 : c;
-    if (!fits) atomicOr(big, 1);
+    rowcnt[r] = c;
+    if (sum > kTileSum || ((c + 3) & ~3u) > (uint32_t)n) atomicOr(big, 1);
   }
 }
 
@@ -137,16 +135,9 @@ __global__ void csr_fill_kernel(const int32_t* __restrict__ A, int m, int n, con
     }
     pos += __popc(bal);
   }
-  const uint32_t q = pos + lane;
-  if (q < rowptr[r + 1]) {  // at most three
-    if (packed) {
-      pack[q] = 0;
-    } else {
-      col[q] = 0;
-      val[q] = 0;
-    }
-  }
   if (!packed) return;
+  const uint32_t q = pos + lane;
+  if (q < rowptr[r + 1]) pack[q] = 0;  // at most three
   for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
   if (lane == 0) start[r] = 0u - 128u * 65537u * sum;
 }
@@ -350,14 +341,15 @@ int prep_lanes(int W) {
 // consecutive words at a time (coalesced): a first sweep sums the segment, the
 // 32 segment sums are scanned by warp 0, and a second sweep scans the
 // segment with warp shuffles and writes it.
-__device__ __forceinline__ void bin_scan_block(const uint32_t* __restrict__ hist, int nbins,
+template <typename Load>
+__device__ __forceinline__ void scan_block(Load hist, int nbins,
                                                uint32_t* __restrict__ start, uint32_t* __restrict__ cursor) {
   __shared__ uint32_t s_warp[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
   const int per = (nbins + nw - 1) / nw;
   const int b0 = wid * per, b1 = min(b0 + per, nbins);
   uint32_t sum = 0;
-  for (int b = b0 + lane; b < b1; b += 32) sum += hist[b];
+  for (int b = b0 + lane; b < b1; b += 32) sum += hist(b);
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) s_warp[wid] = sum;
   __syncthreads();
@@ -373,7 +365,7 @@ __device__ __forceinline__ void bin_scan_block(const uint32_t* __restrict__ hist
   uint32_t run = wid > 0 ? s_warp[wid - 1] : 0;  // exclusive start of the segment
   for (int base = b0; base < b1; base += 32) {
     const int b = base + lane;
-    const uint32_t v = b < b1 ? hist[b] : 0;
+    const uint32_t v = b < b1 ? hist(b) : 0;
     uint32_t x = v;
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -387,9 +379,22 @@ __device__ __forceinline__ void bin_scan_block(const uint32_t* __restrict__ hist
   }
 }
 
+__device__ __forceinline__ void bin_scan_block(const uint32_t* __restrict__ hist, int nbins,
+                                               uint32_t* __restrict__ start, uint32_t* __restrict__ cursor) {
+  scan_block([&](int b) { return hist[b]; }, nbins, start, cursor);
+}
+
 __global__ void bin_scan_kernel(const uint32_t* __restrict__ hist, int nbins, uint32_t* __restrict__ start,
                                 uint32_t* __restrict__ cursor) {
   bin_scan_block(hist, nbins, start, cursor);
+}
+
+// row starts of A in compressed rows: of its nonzeros, or of rows filled up to
+// multiples of four for the tile kernel
+__global__ void csr_scan_kernel(const uint32_t* __restrict__ rowcnt, int m, const int32_t* __restrict__ big,
+                                uint32_t* __restrict__ rowptr) {
+  const uint32_t fill = *big == 0 ? 3u : 0u;
+  scan_block([&](int r) { return (rowcnt[r] + fill) & ~fill; }, m + 1, rowptr, rowptr);
 }
 
 // sorted arrays: row index, folded signatures, l1
@@ -923,8 +928,8 @@ extern "C" int mape_kernel_test(const int32_t* A, int32_t m, int32_t n, const in
     MAPE_CUDA_TRY(cudaMemsetAsync(rowcnt, 0, sizeof(uint32_t) * ((size_t)m + 1), st));
     int32_t* big = reinterpret_cast<int32_t*>(d_fail + 1);
     mape_detail::launch(csr_count_kernel, gw, 256, 0, st, A, m, n, rowcnt, big);
-    // exclusive prefix over m + 1 entries: entry m = nnz(A)
-    mape_detail::launch(bin_scan_kernel, 1, 1024, 0, st, rowcnt, m + 1, rowptr, rowptr);
+    // exclusive prefix over m + 1 entries: entry m = nnz(A) (or that of the filled rows)
+    mape_detail::launch(csr_scan_kernel, 1, 1024, 0, st, rowcnt, m, big, rowptr);
     uint32_t* pack = reinterpret_cast<uint32_t*>(val);
     mape_detail::launch(csr_fill_kernel, gw, 256, 0, st, A, m, n, rowptr, col, val, big, pack, rowcnt);
     // the device decides which of the two kernels works, the call does not wait for it
