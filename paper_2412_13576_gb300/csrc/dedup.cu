@@ -114,7 +114,7 @@ __global__ void compact_reps_kernel(const uint8_t* __restrict__ is_rep, int64_t 
 // Prefix code of a signed byte, order-preserving: codes compare as bit strings
 // (first bit most significant) as the bytes do.  Zero is 10; a positive m is
 // 11 and the code of its magnitude, a negative one 0 and that code inverted.
-// Magnitudes: 0 (1), 10 (2), 110 (3), then 3 + k ones, a zero and k bits for
+// Magnitudes: 0 (1), 10 (2), 110 (3), then k + 1 ones, a zero and k bits for
 // [2^k, 2^(k+1)), k = 2 .. 5, and seven ones and 7 bits from 64 on.  Length in the
 // upper half, bits (right-aligned) in the lower.
 __device__ __forceinline__ uint32_t byte_code(int v) {
@@ -375,6 +375,7 @@ namespace mape_detail {
 
 // Sorts the K pairs of the view; the buffer that holds the result.
 int sort_pairs(const SortView& d, cudaStream_t st) {
+  if (d.K < 2) return 0;  // every row the same: 5 us of 90 for 3000 rows
   const unsigned tiles = (unsigned)ceil_div(d.K, kSortTile);
   launch(sort_tiles_kernel, tiles, kSortThreads, 0, st, d);
   int from = 0;
