@@ -63,6 +63,19 @@ __global__ void __launch_bounds__(kGramThreads) gram_kernel(const int32_t* __res
   }
 }
 
+// The same for small n, a thread per entry over all rows, eight loads at once:
+// the list's barriers outweigh its gain (n = 20: 3.7 us against 5.4)
+constexpr int kGramSmall = 128;
+__global__ void gram_small_kernel(const int32_t* __restrict__ B, int n, int d, float* __restrict__ H) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+  if (j >= d || j < k) return;  // lower triangle: row j >= column k
+  long long acc = 0;
+#pragma unroll 8
+  for (int i = 0; i < n; ++i) acc += (long long)B[(int64_t)i * d + j] * B[(int64_t)i * d + k];
+  H[(int64_t)j * d + k] = (float)acc;
+  H[(int64_t)k * d + j] = (float)acc;
+}
+
 // Blocked right-looking Cholesky of the lower triangle of H (row-major,
 // d x d), panel width kNB: per panel, (1) the diagonal block is factored in
 // shared memory by one CTA, (2) the rows below it are solved against it
@@ -228,6 +241,9 @@ constexpr int kSolveRing = 8;  // rows of L ahead, at most
 
 __host__ __device__ inline size_t solve_row_bytes(int d) { return ((size_t)d * 4 + 15) / 16 * 16; }
 
+// kTail: terms of a lane that the last batch of a step may have, 2 while d <= 64
+// (16 predicated ones a step were most of the instructions at d = 15)
+template <int kTail>
 __global__ void __launch_bounds__(32 * kSolveWarps) w_solve_kernel(const int32_t* __restrict__ B, const float* __restrict__ L,
                                                           const float* __restrict__ Lt, int n, int d, int ring,
                                                           float* __restrict__ W) {
@@ -298,16 +314,16 @@ __global__ void __launch_bounds__(32 * kSolveWarps) w_solve_kernel(const int32_t
           for (int q = 0; q < kSolveRows; ++q) part[q] = fmaf(l[e], v[q][e], part[q]);
       }
       {
-        float l[kSolveBatch], v[kSolveRows][kSolveBatch];
+        float l[kTail], v[kSolveRows][kTail];
 #pragma unroll
-        for (int e = 0; e < kSolveBatch; ++e) {  // the rest; an absent term is skipped, not added as 0
+        for (int e = 0; e < kTail; ++e) {  // the rest; an absent term is skipped, not added as 0
           const bool in = k + 32 * e < ke;
           l[e] = in ? row[k + 32 * e] : 0.f;
 #pragma unroll
           for (int q = 0; q < kSolveRows; ++q) v[q][e] = in ? u[q][k + 32 * e] : 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < kSolveBatch; ++e)
+        for (int e = 0; e < kTail; ++e)
 #pragma unroll
           for (int q = 0; q < kSolveRows; ++q)
             if (k + 32 * e < ke) part[q] = fmaf(l[e], v[q][e], part[q]);
@@ -431,7 +447,10 @@ extern "C" int mape_project_prepare(const int32_t* B, int32_t n, int32_t d, floa
   if (!cv.ok) return MAPE_ERR_CAPACITY;
   cudaStream_t st = as_stream(stream);
   MAPE_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
-  mape_detail::launch(gram_kernel, (unsigned)d, kGramThreads, 0, st, B, n, d, H);
+  if (n <= kGramSmall)
+    mape_detail::launch(gram_small_kernel, dim3((unsigned)ceil_div(d, 128), (unsigned)d), 128, 0, st, B, n, d, H);
+  else
+    mape_detail::launch(gram_kernel, (unsigned)d, kGramThreads, 0, st, B, n, d, H);
   for (int k0 = 0; k0 < d; k0 += kNB) {
     mape_detail::launch(chol_diag_kernel, 1, kNB * kRowThreads, 0, st, H, d, k0, status);
     const int rest = d - k0 - kNB;
@@ -445,14 +464,15 @@ extern "C" int mape_project_prepare(const int32_t* B, int32_t n, int32_t d, floa
   const unsigned g32 = (unsigned)ceil_div(d, 32);
   mape_detail::launch(transpose_lower_kernel, dim3(g32, g32), dim3(32, 8), 0, st, H, d, Lt);
   size_t lim = 0;
-  const int rc = allow_max_dynamic_smem((const void*)w_solve_kernel, &lim);
+  const auto solve = d <= 64 ? w_solve_kernel<2> : w_solve_kernel<kSolveBatch>;
+  const int rc = allow_max_dynamic_smem((const void*)solve, &lim);
   if (rc != MAPE_OK) return rc;
   // the vectors of the block's rows, and as many rows of L ahead as fit
   const size_t rb = solve_row_bytes(d), vecs = (size_t)kSolveWarps * kSolveRows * rb;
   const int ring = vecs + kSolveRing * rb <= lim ? kSolveRing : vecs + 4 * rb <= lim ? 4 : 2;
   const size_t smem = vecs + (size_t)ring * rb;
   if (smem > lim) return MAPE_ERR_SHAPE;
-  mape_detail::launch(w_solve_kernel, (unsigned)ceil_div(n, kSolveWarps * kSolveRows), 32 * kSolveWarps, smem, st, B, H, Lt,
+  mape_detail::launch(solve, (unsigned)ceil_div(n, kSolveWarps * kSolveRows), 32 * kSolveWarps, smem, st, B, H, Lt,
                       n, d, ring, W);
   MAPE_LAUNCH_CHECK();
   int32_t h_status = 0;
