@@ -105,11 +105,13 @@ extern "C" {
  * implementation and the streamed kernels' N-block widths (64, 128 or 256
  * rows of B per forward CTA, coordinates per gradient CTA) for this shape
  * (into MAPE_PREC_FP8: the widths of its streamed kernels only): the
- * first call for a (n, d, P rounded up to a power of two, precision) times a
+ * first call for a (n, d, P rounded up to a power of two, precision), apart for
+ * an identity-topped and a general B and for launch timing off and on, times a
  * few steps of every candidate on scratch copies of the call's state (inside
  * the workspace, which is larger with this bit) and keeps the fastest for the
- * process; later calls reuse it.  Results are those of the chosen
- * implementation; mape_autotune_lookup reports the choice and the probes. */
+ * process; later calls reuse it (the widths 256 and 256 stand for the streamed
+ * default, with an identity-topped B the one launch).  Results are those of the
+ * chosen implementation; mape_autotune_lookup reports the choice and the probes. */
 #define MAPE_PREC_AUTOTUNE 0x200
 /* OR-ing MAPE_PREC_SPARSE_FWD into MAPE_PREC_BF16 runs the forward product
  * of the streamed path on the CUDA cores over the compressed rows of Bm, for
@@ -260,7 +262,8 @@ typedef struct {
   int32_t cand_path[16], cand_wF[16], cand_wG[16];
   float probe_ms[16];       /* their times                                    */
 } mape_tune_info;
-/* The autotuned choice for a shape, or STATE if none was made yet. */
+/* The autotuned choice for a shape (for an identity-topped B with launch timing
+ * off, or else for what was tuned), or STATE if none was made yet. */
 int mape_autotune_lookup(int32_t n, int32_t d, int32_t P, int32_t precision, mape_tune_info* out);
 /* Forgets every autotuned choice of the process (extraction paths and the
  * lane counts of the augmentation scoring pass). */

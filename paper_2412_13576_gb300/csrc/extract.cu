@@ -10,6 +10,7 @@
 #include <cstring>
 #include <atomic>
 #include <mutex>
+#include <tuple>
 #include <vector>
 
 namespace mape_detail {
@@ -150,13 +151,13 @@ bool valid_precision(int32_t precision) {
 
 // ---- autotuning of the implementation (BF16) and the streamed tile widths (BF16, FP8) ----
 
+// The default streamed implementation runs in other kernels for a general B and
+// while launch timing is on, so a choice holds for its kind of call only.
 struct TuneKey {
   int32_t n, d, pb, base;
+  bool general, timed;
   bool operator<(const TuneKey& o) const {
-    if (n != o.n) return n < o.n;
-    if (d != o.d) return d < o.d;
-    if (pb != o.pb) return pb < o.pb;
-    return base < o.base;
+    return std::tie(n, d, pb, base, general, timed) < std::tie(o.n, o.d, o.pb, o.base, o.general, o.timed);
   }
 };
 
@@ -181,19 +182,20 @@ size_t tune_scratch_bytes(int32_t n, int32_t d, int32_t P) {
   return s.bytes();
 }
 
-int run_choice(const mape_extract_args* a, cudaStream_t st, const mape_tune_info& c) {
-  if (c.path == 0) return mape_detail::extract_tc(a, st);
+int run_choice(const mape_extract_args* a, cudaStream_t st, const mape_tune_info& c, mape_detail::Basis basis) {
+  if (c.path == 0) return mape_detail::extract_tc(a, st, basis);
   // the widest blocks stand for the default implementation
-  if (c.path == 1 && c.wF == 256 && c.wG == 256) return mape_detail::extract_stream(a, st, mape_detail::kFwdDense);
-  return mape_detail::extract_stream_widths(a, st, c.wF, c.wG,
-                                            c.path == 2 ? mape_detail::kFwdSparse : mape_detail::kFwdDense);
+  if (c.path == 1 && c.wF == 256 && c.wG == 256) return mape_detail::extract_stream(a, st, mape_detail::kFwdDense, basis);
+  return mape_detail::extract_stream_widths(
+      a, st, c.wF, c.wG, c.path == 2 ? mape_detail::kFwdSparse : mape_detail::kFwdDense, basis);
 }
 
 }  // namespace
 
 // Times kProbeSteps steps of every candidate from the call's state on scratch
 // copies (the call's own arrays are not touched) and caches the fastest.
-static int autotune(const mape_extract_args* a, cudaStream_t st, size_t impl_bytes, mape_tune_info& out) {
+static int autotune(const mape_extract_args* a, cudaStream_t st, size_t impl_bytes, mape_detail::Basis basis,
+                    mape_tune_info& out) {
   using namespace mape_detail;
   const int n = a->n, d = a->d, P = a->P;
   const size_t ldc = align_up((size_t)n, 16);
@@ -246,7 +248,7 @@ static int autotune(const mape_extract_args* a, cudaStream_t st, size_t impl_byt
       MAPE_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
       MAPE_CUDA_TRY(cudaMemsetAsync(fl, 0, sizeof(int32_t), st));
       MAPE_CUDA_TRY(cudaEventRecord(e0, st));
-      rc = run_choice(&b, st, k);
+      rc = run_choice(&b, st, k, basis);
       MAPE_CUDA_TRY(cudaEventRecord(e1, st));
       MAPE_CUDA_TRY(cudaEventSynchronize(e1));
       MAPE_CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
@@ -271,10 +273,15 @@ static int autotune(const mape_extract_args* a, cudaStream_t st, size_t impl_byt
 extern "C" int mape_autotune_lookup(int32_t n, int32_t d, int32_t P, int32_t precision, mape_tune_info* out) {
   if (!out) return MAPE_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  auto it = g_tuned.find(TuneKey{n, d, p_bucket(P), precision & MAPE_PREC_MASK});
-  if (it == g_tuned.end()) return MAPE_ERR_STATE;
-  *out = it->second;
-  return MAPE_OK;
+  // of the shape's choices the one for the usual call: an identity-topped B, untimed
+  for (const bool timed : {false, true})
+    for (const bool general : {false, true}) {
+      auto it = g_tuned.find(TuneKey{n, d, p_bucket(P), precision & MAPE_PREC_MASK, general, timed});
+      if (it == g_tuned.end()) continue;
+      *out = it->second;
+      return MAPE_OK;
+    }
+  return MAPE_ERR_STATE;
 }
 
 extern "C" void mape_autotune_clear(void) {
@@ -336,7 +343,12 @@ extern "C" int mape_extract(const mape_extract_args* a, void* stream) {
       return mape_detail::extract_stream(&b, st, mape_detail::kFwdDense);
     if (a->precision & MAPE_PREC_AUTOTUNE) {
       const size_t impl = mape_detail::align_up(mape_extract_workspace_bytes(a->n, a->d, a->P, base), 256);
-      const TuneKey key{a->n, a->d, p_bucket(a->P), base};
+      int32_t* flag = mape_detail::Carver(a->workspace, a->workspace_bytes).take<int32_t>(1);
+      std::vector<bool> ids;
+      int rc = mape_detail::identity_tops(&a, 1, flag, st, ids);
+      if (rc != MAPE_OK) return rc;
+      const mape_detail::Basis basis = ids[0] ? mape_detail::kBasisIdentity : mape_detail::kBasisGeneral;
+      const TuneKey key{a->n, a->d, p_bucket(a->P), base, !ids[0], mape_detail::launch_timing_on()};
       mape_tune_info choice{};
       bool have = false;
       {
@@ -345,13 +357,12 @@ extern "C" int mape_extract(const mape_extract_args* a, void* stream) {
         if (it != g_tuned.end()) { choice = it->second; have = true; }
       }
       if (!have) {
-        int rc = autotune(a, st, impl, choice);
-        if (rc != MAPE_OK) return rc;
+        if ((rc = autotune(a, st, impl, basis, choice)) != MAPE_OK) return rc;
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_tuned[key] = choice;
       }
       b.workspace_bytes = impl;
-      return run_choice(&b, st, choice);
+      return run_choice(&b, st, choice, basis);
     }
     if (a->precision & MAPE_PREC_SPARSE_FWD) return mape_detail::extract_stream(&b, st, mape_detail::kFwdSparse);
     if (!(a->precision & MAPE_PREC_STREAMED) && mape_detail::extract_tc_supported(a->n, a->d, base)) {

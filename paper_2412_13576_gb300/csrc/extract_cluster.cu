@@ -1284,19 +1284,25 @@ static int launch_clusters(void (*kernel)(KArgs...), int64_t clusters, int C, in
 
 // One call.  *general = true (and nothing done) when B has no identity top, or
 // the step-by-step kernels are faster.
-int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general) {
+int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general, Basis* basis) {
   *general = false;
   if (a->T > kBiasSteps) return MAPE_ERR_SHAPE;
   ClChoice choice;
-  if (a->d >= a->n || !cl_choose(a, ceil_div(a->P, kTM), &choice)) { *general = true; return MAPE_OK; }
+  if (a->d >= a->n || *basis == kBasisGeneral || !cl_choose(a, ceil_div(a->P, kTM), &choice)) {
+    *general = true;
+    return MAPE_OK;
+  }
   Carver cv(a->workspace, a->workspace_bytes);
   ClCarved c;
   cl_carve(cv, cl_shape(a->n, a->d, a->P), a->precision, &c);
   if (!cv.ok) return MAPE_ERR_CAPACITY;
-  std::vector<bool> ids;
-  int rc = identity_tops(&a, 1, c.hflags, st, ids);
-  if (rc != MAPE_OK) return rc;
-  if (!ids[0]) { *general = true; return MAPE_OK; }
+  int rc;
+  if (*basis == kBasisUnknown) {
+    std::vector<bool> ids;
+    if ((rc = identity_tops(&a, 1, c.hflags, st, ids)) != MAPE_OK) return rc;
+    *basis = ids[0] ? kBasisIdentity : kBasisGeneral;
+  }
+  if (*basis == kBasisGeneral) { *general = true; return MAPE_OK; }
   ClParams p;
   cl_params(c, a, choice, p);
   if ((rc = cl_pack(p, a, c.hflags + 1, st)) != MAPE_OK) return rc;

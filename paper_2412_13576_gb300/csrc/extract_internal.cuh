@@ -13,7 +13,10 @@ int extract_fp32(const mape_extract_args* a, cudaStream_t st);
 
 size_t extract_tc_workspace(int32_t n, int32_t d, int32_t P, int32_t precision);
 bool extract_tc_supported(int32_t n, int32_t d, int32_t precision);
-int extract_tc(const mape_extract_args* a, cudaStream_t st);
+// Whether the top d x d block of B is the identity: tested by the call itself
+// (an extra launch and wait), unless the caller has done so.
+enum Basis { kBasisUnknown = -1, kBasisGeneral = 0, kBasisIdentity = 1 };
+int extract_tc(const mape_extract_args* a, cudaStream_t st, Basis basis = kBasisUnknown);
 
 // Batches of calls (same T, t0, period, precision) on the resident kernel:
 // prepare uploads and synchronises; enqueue only launches kernels.
@@ -35,15 +38,16 @@ size_t extract_stream_workspace(int32_t n, int32_t d, int32_t P);
 // sparse forward (SHAPE unless B is identity-topped, z is carried in full
 // and Bm has density at most 1/16)
 constexpr int kFwdDense = 1, kFwdSparse = 2;
-int extract_stream(const mape_extract_args* a, cudaStream_t st, int fwd_mode);
+int extract_stream(const mape_extract_args* a, cudaStream_t st, int fwd_mode, Basis basis = kBasisUnknown);
 // the same with the forward and gradient N-block widths chosen (64..256, multiples of 64)
-int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, int wG, int fwd_mode);
+int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, int wG, int fwd_mode,
+                          Basis basis = kBasisUnknown);
 
 // the same for an identity-topped B in one launch of tile clusters
 // (extract_cluster.cu); *general = true, and nothing done, for another B and
-// where the step-by-step kernels are faster
+// where the step-by-step kernels are faster; *basis as far as it was found out
 size_t extract_cluster_workspace(int32_t n, int32_t d, int32_t P, int32_t precision);
-int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general);
+int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general, Basis* basis);
 // and for a batch of such calls (same T, t0, period, precision)
 struct ClBatch;
 size_t extract_cluster_batch_workspace(const mape_extract_args* const* items, int count);

@@ -1276,19 +1276,18 @@ static void st_schedule(int t0, int T, int period, Fwd fwd, Coll coll, Grad grad
   }
 }
 
-int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, int wG, int fwd_mode) {
+int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, int wG, int fwd_mode, Basis basis) {
   const int d = a->d, P = a->P;
   if (wF < kKC || wF > kNB || wF % kKC || wG < kKC || wG > kNB || wG % kKC) return MAPE_ERR_INVALID_ARG;
   StCarved c;
   int rc = st_carve(a, false, c);
   if (rc != MAPE_OK) return rc;
-  MAPE_CUDA_TRY(cudaMemsetAsync(c.hflags, 0, sizeof(int32_t), st));
-  launch(stream_identity_top_kernel, (unsigned)ceil_div((int64_t)d * d, 256), 256, 0, st, a->B, d, c.hflags);
-  MAPE_LAUNCH_CHECK();
-  int32_t h_notid = 1;
-  MAPE_CUDA_TRY(cudaMemcpyAsync(&h_notid, c.hflags, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  MAPE_CUDA_TRY(cudaStreamSynchronize(st));
-  const bool id = h_notid == 0;
+  if (basis == kBasisUnknown) {
+    std::vector<bool> ids;
+    if ((rc = identity_tops(&a, 1, c.hflags, st, ids)) != MAPE_OK) return rc;
+    basis = ids[0] ? kBasisIdentity : kBasisGeneral;
+  }
+  const bool id = basis == kBasisIdentity;
   c.sh = stream_shape(a->n, d, P, id, wF, wG);
   if ((rc = st_pack_b(c, a, st)) != MAPE_OK) return rc;
   // the sparse forward: asked for, an identity-topped B, z carried in full
@@ -1430,13 +1429,13 @@ int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, i
 // there names, the step-by-step kernels at their widest blocks for those, for a
 // general B, for the sparse forward, and while launch timing is on, whose kinds
 // are those kernels.  The same bits either way.
-int extract_stream(const mape_extract_args* a, cudaStream_t st, int fwd_mode) {
+int extract_stream(const mape_extract_args* a, cudaStream_t st, int fwd_mode, Basis basis) {
   if (fwd_mode == kFwdDense && !launch_timing_on()) {
     bool general = false;
-    const int rc = extract_cluster(a, st, &general);
+    const int rc = extract_cluster(a, st, &general, &basis);
     if (rc != MAPE_OK || !general) return rc;
   }
-  return extract_stream_widths(a, st, kNB, kNB, fwd_mode);
+  return extract_stream_widths(a, st, kNB, kNB, fwd_mode, basis);
 }
 
 struct StBatch {

@@ -1144,7 +1144,7 @@ static int tc_unpack(const TcParams& p, const mape_extract_args* a, cudaStream_t
 // fit in 512 columns
 static bool tc_resident_state(const TcParams& p) { return 3 * p.d_pad <= kTmemCols; }
 
-int extract_tc(const mape_extract_args* a, cudaStream_t st) {
+int extract_tc(const mape_extract_args* a, cudaStream_t st, Basis basis) {
   const int d = a->d;
   if (a->T > (1 << 20)) return MAPE_ERR_SHAPE;
   // which kernel: identity-topped B or general B (the flag word is the
@@ -1155,13 +1155,16 @@ int extract_tc(const mape_extract_args* a, cudaStream_t st) {
   cv.take<float2>((size_t)1 << 20);
   int32_t* idflag = cv.take<int32_t>(1);
   if (!cv.ok) return MAPE_ERR_CAPACITY;
-  MAPE_CUDA_TRY(cudaMemsetAsync(idflag, 0, sizeof(int32_t), st));
-  mape_detail::launch(identity_top_kernel, (unsigned)ceil_div((int64_t)d * d, 256), 256, 0, st, a->B, d, idflag);
-  MAPE_LAUNCH_CHECK();
-  int32_t h_notid = 1;
-  MAPE_CUDA_TRY(cudaMemcpyAsync(&h_notid, idflag, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  MAPE_CUDA_TRY(cudaStreamSynchronize(st));
-  const bool id = h_notid == 0;
+  if (basis == kBasisUnknown) {
+    MAPE_CUDA_TRY(cudaMemsetAsync(idflag, 0, sizeof(int32_t), st));
+    mape_detail::launch(identity_top_kernel, (unsigned)ceil_div((int64_t)d * d, 256), 256, 0, st, a->B, d, idflag);
+    MAPE_LAUNCH_CHECK();
+    int32_t h_notid = 1;
+    MAPE_CUDA_TRY(cudaMemcpyAsync(&h_notid, idflag, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    MAPE_CUDA_TRY(cudaStreamSynchronize(st));
+    basis = h_notid == 0 ? kBasisIdentity : kBasisGeneral;
+  }
+  const bool id = basis == kBasisIdentity;
   TcParams p;
   uint32_t smem = 0;
   int rc = tc_prepare(a, id, st, p, smem);
