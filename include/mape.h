@@ -202,9 +202,9 @@ typedef struct {
   const int32_t* span;     /* [n] int32, u - l (C4), each in [0, 127]: device  */
                            /* memory, not checked by this call (a larger span  */
                            /* lets values beyond int8 into the candidate rows) */
-  float* Z;                /* [P x d] in/out                                  */
-  float* M;                /* [P x d] in/out, Adam first moment               */
-  float* V;                /* [P x d] in/out, Adam second moment              */
+  float* Z;                /* [P x d] in/out; scratch while the call runs,    */
+  float* M;                /* [P x d]   as are M, the Adam first moment,      */
+  float* V;                /* [P x d]   and V, the second                     */
   int32_t t0, T, period, precision;
   float lambda1, lambda2, lr, eps;
   double beta1, beta2;
@@ -221,7 +221,9 @@ typedef struct {
                               4 = on the FP32 path, |round(z)| above
                               (2^24 - 1) / max_i sum_j |B_ij|, beyond which
                               B round(z) is not exact in FP32 (that start's
-                              rounding is not collected)                 */
+                              rounding is not collected),
+                              16 = a wait within a kernel ran out of its
+                              time: the call's results are void            */
   float* dbg_phi;          /* optional [P]: Phi at the input point            */
   float* dbg_grad;         /* optional [P x d]: gradient at the input point   */
   void* workspace;

@@ -85,19 +85,26 @@ constexpr uint32_t kSbo16 = 512, kSbo8 = 256;
 
 struct ClParams {
   int n, d, P, R;       // R: rows of Bm = n - d
-  int d32, R32, d64;    // padded to 32; d64: pitch of the blocked state
+  int d32, R32;         // padded to 32
   int tiles, C, dyn;    // blocks per cluster; dynamic shared memory of a block
-  int ldc, mapoff, lds; // candidate pitch; offset of the Bm rows in a staged row; its pitch
+  int ldc, ldi;         // candidate pitch; pitch of the staged identity rows
   const uint8_t* Bf;    // forward operand: per block and 128-row block, [d32/32][rows x 32] chunks
   const uint8_t* Bf8;   // the same in e4m3
   const uint8_t* Bg;    // gradient operand: per block and 256-coordinate block, [R32/32][coordinates x 32]
   const int32_t* span;
   float* Zt;
   float* Mt;
-  float* Vt;            // blocked [tiles][d64/4][128][4]
-  uint8_t* Zh;          // z operands (z_tile)
+  float* Vt;            // blocked [tiles][d32/4][128][4]
+  // z operands (z_tile): tiles below z1 at Zh[0], the next up to z2 at Zh[1],
+  // the rest at Zh[2]
+  uint8_t* Zh[3];
+  int z1, z2;
+  int z_out;            // 1: they lie in the caller's M, V and Z
   uint8_t* S;           // [tiles][R32/32] chunks
-  int8_t* stage;        // [2][tiles*128][lds] staged candidate rows, by step parity
+  // staged candidate rows: the identity rows [2][tiles*128][ldi] by step parity
+  // (those of a step are written while the last step's are read), the Bm rows
+  // [tiles*128][R32] (written before a step's gradient, read during it)
+  int8_t *stage, *stage_map;
   unsigned long long* zkey;  // [2][tiles*128]: (|z|_inf bits << 32) | (~first argmax)
   uint32_t* acc;        // [2][..] rounding changed / unexact since the last collection
   uint32_t* oob;        // Bm rows of the staged candidate out of the box
@@ -185,7 +192,10 @@ __device__ __forceinline__ uint32_t z_stride(const ClParams& p) {
   return z_bytes(p) + (p.period == 1 ? (uint32_t)kChunk16 : 0u);
 }
 __device__ __forceinline__ uint8_t* z_tile(const ClParams& p, int tile) {
-  return p.Zh + (size_t)tile * (p.d32 / kKC) * (z_bytes(p) + kChunk16);
+  const size_t bytes = (size_t)(p.d32 / kKC) * (z_bytes(p) + kChunk16);
+  if (tile < p.z1) return p.Zh[0] + tile * bytes;
+  if (tile < p.z2) return p.Zh[1] + (tile - p.z1) * bytes;
+  return p.Zh[2] + (tile - p.z2) * bytes;
 }
 
 // the BF16 operand words of 8 coordinates: hi, and lo = bf16(z - hi)
@@ -200,9 +210,9 @@ __device__ __forceinline__ void split8(const float (&z)[8], uint32_t (&wh)[4], u
 
 // A candidate row of start pg from its staged row, in canonical sign, by the
 // calling warp: 4 bytes per lane where the pieces are aligned
-__device__ __forceinline__ void write_row(const ClParams& p, const int8_t* src, int8_t* dst, bool neg) {
+__device__ __forceinline__ void write_row(const ClParams& p, const int8_t* src, const int8_t* map, int8_t* dst, bool neg) {
   const int lane = threadIdx.x & 31;
-  const int d = p.d, n = p.n, mo = p.mapoff;
+  const int d = p.d, n = p.n;
   const bool words = (reinterpret_cast<uintptr_t>(dst) & 3) == 0;
 #pragma unroll 1
   for (int b = 4 * lane; b < p.ldc; b += 128) {
@@ -210,13 +220,13 @@ __device__ __forceinline__ void write_row(const ClParams& p, const int8_t* src, 
     if (b + 4 <= d) {
       v = __ldcg(reinterpret_cast<const unsigned int*>(src + b));
     } else if (b >= d && (d & 3) == 0 && b + 4 <= n) {
-      v = __ldcg(reinterpret_cast<const unsigned int*>(src + mo + (b - d)));
+      v = __ldcg(reinterpret_cast<const unsigned int*>(map + (b - d)));
     } else {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int i = b + k;
         if (i < n) {
-          const int8_t x = (int8_t)__ldcg(reinterpret_cast<const signed char*>(src + (i < d ? i : mo + (i - d))));
+          const int8_t x = (int8_t)__ldcg(reinterpret_cast<const signed char*>(i < d ? src + i : map + (i - d)));
           v |= (uint32_t)(uint8_t)x << (8 * k);
         }
       }
@@ -281,9 +291,9 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
   const int64_t pg = (int64_t)tile * kTM + r;
   const bool row_live = pg < p.P;
   const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-  float4* const zt = reinterpret_cast<float4*>(p.Zt) + (size_t)tile * (p.d64 / 4) * kTM + r;
-  float4* const mt = reinterpret_cast<float4*>(p.Mt) + (size_t)tile * (p.d64 / 4) * kTM + r;
-  float4* const vt = reinterpret_cast<float4*>(p.Vt) + (size_t)tile * (p.d64 / 4) * kTM + r;
+  float4* const zt = reinterpret_cast<float4*>(p.Zt) + (size_t)tile * (p.d32 / 4) * kTM + r;
+  float4* const mt = reinterpret_cast<float4*>(p.Mt) + (size_t)tile * (p.d32 / 4) * kTM + r;
+  float4* const vt = reinterpret_cast<float4*>(p.Vt) + (size_t)tile * (p.d32 / 4) * kTM + r;
   const uint32_t zstride = z_stride(p), zbytes = z_bytes(p);
   uint8_t* const zh = z_tile(p, tile);
   uint8_t* const zr = zh + (p.period == 1 ? zbytes : nkF * zbytes);
@@ -397,7 +407,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
   // arrays) into its stage, by one lane of the calling warp
   auto load_state = [&](int ch) {
     const uint32_t e = ec + (uint32_t)ch, st = e % kEStages;
-    const size_t o = ((size_t)tile * p.d64 + col0 + ch * 8) * kTM;
+    const size_t o = ((size_t)tile * p.d32 + col0 + ch * 8) * kTM;
     const uint32_t dst = ering + st * kEBytes, bar = efull0 + 8 * st;
     mbar_expect_tx_if(lead, bar, kEBytes);
     bulk_g2s_if(lead, dst, p.Zt + o, kEArr, bar);
@@ -575,7 +585,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
                 pk[k >> 2] |= ((uint32_t)(gv & 0xff)) << (8 * (k & 3));
               }
               if (row_live)
-                *reinterpret_cast<uint4*>(p.stage + ((s & 1) * P2 + pg) * p.lds + p.mapoff + i0) =
+                *reinterpret_cast<uint4*>(p.stage_map + pg * p.R32 + i0) =
                     make_uint4(pk[0], pk[1], pk[2], pk[3]);
             }
           }
@@ -673,7 +683,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
         const long long sl = __shfl_sync(0xffffffffu, slot, l);
         const int ng = __shfl_sync(0xffffffffu, neg, l);
         const int64_t ps = (int64_t)tile * kTM + rank * per + (warp - 2) * mine + l;
-        write_row(p, p.stage + ((s & 1) * P2 + ps) * p.lds, p.cand + sl * p.ldc, ng != 0);
+        write_row(p, p.stage + ((s & 1) * P2 + ps) * p.ldi, p.stage_map + ps * p.R32, p.cand + sl * p.ldc, ng != 0);
       }
     }
     if (!do_fwd) break;
@@ -695,7 +705,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
       float dsum = 0.f;  // sum of |rint(z_new) - rint(z_old)|: 0 iff no rounding changed
       int nkmax = -1, first_id = kNoNz;  // the first maximiser of |z|; the first nonzero rounding
       bool out_id = false, nan_head = false;
-      int8_t* srow = p.stage + (((s + 1) & 1) * P2 + pg) * p.lds;
+      int8_t* srow = p.stage + (((s + 1) & 1) * P2 + pg) * p.ldi;
 #pragma unroll 1
       for (int cb = 0; cb < CS; cb += kColBlk) {
         const int nch = (CS - cb < kColBlk ? CS - cb : kColBlk) / 8;
@@ -846,7 +856,7 @@ __device__ __forceinline__ void cluster_body(const ClParams& p, const int tile, 
               for (int k = 7; k >= 0; --k)
                 if (rn[k] != 0.f) first_id = ((j0 + k) << 1) | (rn[k] < 0.f ? 1 : 0);
             }
-            if (row_live && j0 < p.mapoff) *reinterpret_cast<uint2*>(srow + j0) = make_uint2(bb[0], bb[1]);
+            if (row_live && j0 < p.ldi) *reinterpret_cast<uint2*>(srow + j0) = make_uint2(bb[0], bb[1]);
           }
           // the stage's next chunk, once the three other warps have read it
           if (q == 0 && cb / 8 + ch + kEStages < CS / 8) {
@@ -971,18 +981,40 @@ __global__ void cl_pack_b_kernel(const int32_t* __restrict__ B, int d, int R, in
 // start at a time (coalesced), shared memory turns them.
 constexpr int kInitRows = 32;
 
+// the operands of z0 from the blocked state, 8 coordinates of a start per thread
+__device__ __forceinline__ void z_operands(const ClParams& p, int tile, int rq) {
+  const int row = rq * kInitRows + (threadIdx.x & 31), part = threadIdx.x >> 5;
+  const size_t base = (size_t)tile * (p.d32 / 4) * kTM + row;
+  const float sc = p.f8 ? scale_of(__ldcg(&p.zkey[(int64_t)tile * kTM + row])) : 1.f;
+  for (int j0 = 8 * part; j0 < p.d32; j0 += 64) {
+    const size_t o = base + (size_t)(j0 / 4) * kTM;
+    const float4 a = reinterpret_cast<const float4*>(p.Zt)[o], b = reinterpret_cast<const float4*>(p.Zt)[o + kTM];
+    uint8_t* const zo = z_tile(p, tile) + (size_t)(j0 >> 5) * z_stride(p);
+    if (p.f8) {
+      const float v8[8] = {a.x * sc, a.y * sc, a.z * sc, a.w * sc, b.x * sc, b.y * sc, b.z * sc, b.w * sc};
+      *reinterpret_cast<uint2*>(zo + off8(row, j0 & 31)) = pack_e4m3x8(v8);
+    } else {
+      const float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+      uint32_t wh[4], wl[4];
+      split8(z, wh, wl);
+      const uint32_t oc = off16(row, j0 & 31);
+      *reinterpret_cast<uint4*>(zo + oc) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+      if (p.nterms > 1) *reinterpret_cast<uint4*>(zo + kChunk16 + oc) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256) cl_init_kernel(ClParams p, const float* __restrict__ Z,
                                                       const float* __restrict__ M, const float* __restrict__ V) {
   __shared__ float t[3][kInitRows][33];
   __shared__ float s_best[kInitRows][8];
   __shared__ int s_at[kInitRows][8];
-  __shared__ float s_sc[kInitRows];
   const int tile = blockIdx.x / (kTM / kInitRows), rq = blockIdx.x % (kTM / kInitRows);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t pg0 = (int64_t)tile * kTM + rq * kInitRows;
   const int64_t P2 = (int64_t)p.tiles * kTM;
   const int rr = tid & 31, part = tid >> 5;  // the turned side: start rr, coordinates 4 part ..
-  const size_t base = (size_t)tile * (p.d64 / 4) * kTM + rq * kInitRows + rr;
+  const size_t base = (size_t)tile * (p.d32 / 4) * kTM + rq * kInitRows + rr;
   float best = 0.f;
   int kb = -1;
   for (int j0 = 0; j0 < p.d32; j0 += 32) {
@@ -1007,19 +1039,6 @@ __global__ void __launch_bounds__(256) cl_init_kernel(ClParams p, const float* _
       const int j = j0 + c + k;
       if (j < p.d && (j == 0 || (kb < 0 ? a == a : a > best))) { best = a; kb = j; }
     }
-    if (!p.f8) {
-      uint32_t wh[2], wl[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const float z0 = t[0][rr][c + 2 * k], z1 = t[0][rr][c + 2 * k + 1];
-        wh[k] = pack_bf16x2(z0, z1);
-        const float2 hf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&wh[k]));
-        wl[k] = pack_bf16x2(z0 - hf.x, z1 - hf.y);
-      }
-      uint8_t* const zo = z_tile(p, tile) + (size_t)(j0 >> 5) * z_stride(p) + off16(rq * kInitRows + rr, c);
-      *reinterpret_cast<uint2*>(zo) = make_uint2(wh[0], wh[1]);
-      if (p.nterms > 1) *reinterpret_cast<uint2*>(zo + kChunk16) = make_uint2(wl[0], wl[1]);
-    }
     __syncthreads();
   }
   s_best[rr][part] = best;
@@ -1036,7 +1055,6 @@ __global__ void __launch_bounds__(256) cl_init_kernel(ClParams p, const float* _
     }
     const unsigned long long key =
         pg < p.P ? ((unsigned long long)__float_as_uint(b) << 32) | (0xffffffffu - (uint32_t)at) : 0ull;
-    s_sc[tid] = scale_of(key);
     p.zkey[pg] = key;
     p.zkey[P2 + pg] = 0ull;
     p.oob[pg] = 0u;
@@ -1047,16 +1065,13 @@ __global__ void __launch_bounds__(256) cl_init_kernel(ClParams p, const float* _
     }
     if (p.dbg_phi && pg < p.P) p.dbg_phi[pg] = 0.f;
   }
-  if (!p.f8) return;
+  if (p.z_out) return;  // other blocks still read where the operands go: cl_operand_kernel
   __syncthreads();
-  const float sc = s_sc[rr];
-  for (int j0 = 8 * part; j0 < p.d32; j0 += 64) {  // e4m3 operand, 8 coordinates of a start per thread
-    const size_t o = base + (size_t)(j0 / 4) * kTM;
-    const float4 a = reinterpret_cast<const float4*>(p.Zt)[o], b = reinterpret_cast<const float4*>(p.Zt)[o + kTM];
-    const float v8[8] = {a.x * sc, a.y * sc, a.z * sc, a.w * sc, b.x * sc, b.y * sc, b.z * sc, b.w * sc};
-    *reinterpret_cast<uint2*>(z_tile(p, tile) + (size_t)(j0 >> 5) * z_stride(p) + off8(rq * kInitRows + rr, j0 & 31)) =
-        pack_e4m3x8(v8);
-  }
+  z_operands(p, tile, rq);
+}
+
+__global__ void __launch_bounds__(256) cl_operand_kernel(ClParams p) {
+  z_operands(p, blockIdx.x / (kTM / kInitRows), blockIdx.x % (kTM / kInitRows));
 }
 
 // the blocked state back to the caller's rows
@@ -1067,7 +1082,7 @@ __global__ void __launch_bounds__(256) cl_unpack_kernel(ClParams p, float* __res
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t pg0 = (int64_t)tile * kTM + rq * kInitRows;
   const int rr = tid & 31, c = 4 * (tid >> 5);
-  const size_t base = (size_t)tile * (p.d64 / 4) * kTM + rq * kInitRows + rr;
+  const size_t base = (size_t)tile * (p.d32 / 4) * kTM + rq * kInitRows + rr;
   for (int j0 = 32 * blockIdx.y; j0 < p.d32; j0 += 32 * gridDim.y) {
     const size_t o = base + (size_t)((j0 + c) / 4) * kTM;
     const float4 z = reinterpret_cast<const float4*>(p.Zt)[o], m = reinterpret_cast<const float4*>(p.Mt)[o],
@@ -1090,23 +1105,35 @@ __global__ void __launch_bounds__(256) cl_unpack_kernel(ClParams p, float* __res
 }
 
 int pad32(int x) { return (x + 31) / 32 * 32; }
-int pad64(int x) { return (x + 63) / 64 * 64; }
 int pad16(int x) { return (x + 15) / 16 * 16; }
 
-constexpr int32_t kBiasSteps = 1 << 20;
+constexpr int32_t kBiasSteps = 1 << 19;  // steps of a call: half of the step-by-step kernels' table, half its bytes
+constexpr size_t kZAlign = 128;
 
+// The z operands lie in the caller's M, V and Z where they fit: from the packing
+// of the state to its unpacking these hold nothing that is needed.  (In the
+// workspace they made it larger than that of the step-by-step kernels, by 31%
+// at n = 2000 and P = 65536, and a server whose memory cap lay between refused
+// the request.)  Where they do not fit, for a few hundred starts, the workspace has
+// room for them.
 struct ClShape {
-  int R, d32, R32, d64, tiles, mapoff, lds;
+  int R, d32, R32, tiles, ldi;
+  size_t z_tile;   // bytes of a tile's z operands
+  int z_fit;       // tiles that fit in each of the three arrays, at any address
+  bool z_out;
 };
-ClShape cl_shape(int n, int d, int P) {
+ClShape cl_shape(int n, int d, int P, int32_t precision) {
   ClShape s{};
   s.R = n - d;
   s.d32 = pad32(d);
   s.R32 = s.R > 0 ? pad32(s.R) : 32;
-  s.d64 = pad64(d);
   s.tiles = (int)mape_detail::ceil_div(P, kTM);
-  s.mapoff = pad16(d);
-  s.lds = s.mapoff + s.R32;
+  s.ldi = pad16(d);
+  const int per = precision == MAPE_PREC_FP8 ? 3 : precision == MAPE_PREC_BF16 ? 6 : 4;  // bytes a coordinate
+  s.z_tile = (size_t)kTM * s.d32 * per;
+  const size_t bytes = sizeof(float) * (size_t)P * d;
+  s.z_fit = bytes > kZAlign ? (int)std::min<size_t>((bytes - kZAlign) / s.z_tile, (size_t)s.tiles) : 0;
+  s.z_out = 3ll * s.z_fit >= s.tiles;
   return s;
 }
 
@@ -1114,7 +1141,7 @@ struct ClCarved {
   ClShape sh;
   float *Zt, *Mt, *Vt;
   uint8_t *Zh, *S, *Bf, *Bg, *Bf8;
-  int8_t* stage;
+  int8_t *stage, *stage_map;
   unsigned long long* zkey;
   uint32_t *acc, *oob, *idw;
   int32_t *first, *hflags;
@@ -1122,9 +1149,8 @@ struct ClCarved {
 };
 
 template <typename Carve>
-void cl_carve(Carve& cv, const ClShape& sh, int32_t precision, ClCarved* c) {
+void cl_carve(Carve& cv, const ClShape& sh, ClCarved* c) {
   const size_t P2 = (size_t)sh.tiles * kTM;
-  const bool f8 = precision == MAPE_PREC_FP8, two = precision == MAPE_PREC_BF16;
   ClCarved k{};
   k.sh = sh;
   auto take = [&](auto*& ptr, size_t count) {
@@ -1132,12 +1158,13 @@ void cl_carve(Carve& cv, const ClShape& sh, int32_t precision, ClCarved* c) {
     if constexpr (std::is_same_v<Carve, mape_detail::Carver>) ptr = cv.template take<T>(count);
     else cv.template take<T>(count);
   };
-  take(k.Zt, P2 * sh.d64);
-  take(k.Mt, P2 * sh.d64);
-  take(k.Vt, P2 * sh.d64);
-  take(k.Zh, P2 * sh.d32 * (f8 ? 3 : two ? 6 : 4));
+  take(k.Zt, P2 * sh.d32);
+  take(k.Mt, P2 * sh.d32);
+  take(k.Vt, P2 * sh.d32);
+  if (!sh.z_out) take(k.Zh, sh.z_tile * sh.tiles);
   take(k.S, P2 * sh.R32 * 2);
-  take(k.stage, 2 * P2 * sh.lds);
+  take(k.stage, 2 * P2 * sh.ldi);
+  take(k.stage_map, P2 * sh.R32);
   take(k.Bf, (size_t)sh.R32 * sh.d32 * 2);
   take(k.Bg, (size_t)sh.R32 * sh.d32 * 2);
   take(k.Bf8, (size_t)sh.R32 * sh.d32);
@@ -1203,20 +1230,33 @@ static bool cl_choose(const mape_extract_args* a, int64_t tiles, ClChoice* c) {
   return true;
 }
 
+bool extract_cluster_takes(const mape_extract_args* a) { return a->d < a->n && a->T <= kBiasSteps; }
+
 size_t extract_cluster_workspace(int32_t n, int32_t d, int32_t P, int32_t precision) {
   if (d >= n) return 0;
   Sizer s;
-  cl_carve(s, cl_shape(n, d, P), precision, nullptr);
+  cl_carve(s, cl_shape(n, d, P, precision), nullptr);
   return s.bytes();
 }
 
 static void cl_params(const ClCarved& c, const mape_extract_args* a, ClChoice choice, ClParams& p) {
   const ClShape& sh = c.sh;
   p = ClParams{};
-  p.n = a->n; p.d = a->d; p.P = a->P; p.R = sh.R; p.d32 = sh.d32; p.R32 = sh.R32; p.d64 = sh.d64;
-  p.tiles = sh.tiles; p.C = choice.C; p.dyn = choice.dyn; p.ldc = a->ldc; p.mapoff = sh.mapoff; p.lds = sh.lds;
+  p.n = a->n; p.d = a->d; p.P = a->P; p.R = sh.R; p.d32 = sh.d32; p.R32 = sh.R32;
+  p.tiles = sh.tiles; p.C = choice.C; p.dyn = choice.dyn; p.ldc = a->ldc; p.ldi = sh.ldi;
   p.Bf = c.Bf; p.Bf8 = c.Bf8; p.Bg = c.Bg; p.span = a->span; p.Zt = c.Zt; p.Mt = c.Mt; p.Vt = c.Vt;
-  p.Zh = c.Zh; p.S = c.S; p.stage = c.stage; p.zkey = c.zkey; p.acc = c.acc;
+  p.z_out = sh.z_out ? 1 : 0;
+  if (sh.z_out) {
+    float* const at[3] = {a->M, a->V, a->Z};
+    for (int k = 0; k < 3; ++k)
+      p.Zh[k] = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(at[k]) + kZAlign - 1) / kZAlign * kZAlign);
+    p.z1 = std::min(sh.z_fit, sh.tiles);
+    p.z2 = std::min(2 * sh.z_fit, sh.tiles);
+  } else {
+    p.Zh[0] = p.Zh[1] = p.Zh[2] = c.Zh;
+    p.z1 = p.z2 = sh.tiles;
+  }
+  p.S = c.S; p.stage = c.stage; p.stage_map = c.stage_map; p.zkey = c.zkey; p.acc = c.acc;
   p.oob = c.oob; p.idw = c.idw; p.first = c.first; p.bias = c.bias;
   p.lambda1 = a->lambda1; p.lambda2 = a->lambda2; p.eps = a->eps;
   p.beta1 = (float)a->beta1; p.beta2 = (float)a->beta2;
@@ -1246,6 +1286,7 @@ static int cl_setup(const ClCarved& c, const ClParams& p, const mape_extract_arg
   MAPE_CUDA_TRY(cudaMemcpyAsync(c.bias, bc.data(), sizeof(float2) * bc.size(), cudaMemcpyHostToDevice, st));
   launch(cl_init_kernel, (unsigned)(p.tiles * (kTM / kInitRows)), 256, 0, st, p, (const float*)a->Z,
          (const float*)a->M, (const float*)a->V);
+  if (p.z_out) launch(cl_operand_kernel, (unsigned)(p.tiles * (kTM / kInitRows)), 256, 0, st, p);
   MAPE_LAUNCH_CHECK();
   return MAPE_OK;
 }
@@ -1286,15 +1327,14 @@ static int launch_clusters(void (*kernel)(KArgs...), int64_t clusters, int C, in
 // the step-by-step kernels are faster.
 int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general, Basis* basis) {
   *general = false;
-  if (a->T > kBiasSteps) return MAPE_ERR_SHAPE;
   ClChoice choice;
-  if (a->d >= a->n || *basis == kBasisGeneral || !cl_choose(a, ceil_div(a->P, kTM), &choice)) {
+  if (!extract_cluster_takes(a) || *basis == kBasisGeneral || !cl_choose(a, ceil_div(a->P, kTM), &choice)) {
     *general = true;
     return MAPE_OK;
   }
   Carver cv(a->workspace, a->workspace_bytes);
   ClCarved c;
-  cl_carve(cv, cl_shape(a->n, a->d, a->P), a->precision, &c);
+  cl_carve(cv, cl_shape(a->n, a->d, a->P, a->precision), &c);
   if (!cv.ok) return MAPE_ERR_CAPACITY;
   int rc;
   if (*basis == kBasisUnknown) {
@@ -1367,9 +1407,8 @@ int extract_cluster_batch_prepare(const mape_extract_args* const* items, int cou
   int rc;
   for (int i = 0; i < count; ++i) {
     const mape_extract_args* a = items[i];
-    if (a->T > kBiasSteps) return MAPE_ERR_SHAPE;
     Carver cv(a->workspace, a->workspace_bytes);
-    cl_carve(cv, cl_shape(a->n, a->d, a->P), a->precision, &carved[i]);
+    cl_carve(cv, cl_shape(a->n, a->d, a->P, a->precision), &carved[i]);
     if (!cv.ok) return MAPE_ERR_CAPACITY;
     // by the tiles of the whole batch: 0.75 to 0.95 of the time of a rule by d
     // alone (8 blocks from 512 coordinates on, 4 from 256, else 2), which for 8

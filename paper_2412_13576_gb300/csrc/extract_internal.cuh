@@ -46,6 +46,7 @@ int extract_stream_widths(const mape_extract_args* a, cudaStream_t st, int wF, i
 // the same for an identity-topped B in one launch of tile clusters
 // (extract_cluster.cu); *general = true, and nothing done, for another B and
 // where the step-by-step kernels are faster; *basis as far as it was found out
+bool extract_cluster_takes(const mape_extract_args* a);  // by its sizes
 size_t extract_cluster_workspace(int32_t n, int32_t d, int32_t P, int32_t precision);
 int extract_cluster(const mape_extract_args* a, cudaStream_t st, bool* general, Basis* basis);
 // and for a batch of such calls (same T, t0, period, precision)

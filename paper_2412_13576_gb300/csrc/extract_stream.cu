@@ -1503,7 +1503,7 @@ int extract_stream_batch_prepare(const mape_extract_args* const* all, const bool
   std::vector<const mape_extract_args*> cl, gen;
   std::vector<char> gen_ids;
   for (int i = 0; i < all_count; ++i) {
-    if (all_ids[i] && all[i]->d < all[i]->n) cl.push_back(all[i]);
+    if (all_ids[i] && extract_cluster_takes(all[i])) cl.push_back(all[i]);
     else { gen.push_back(all[i]); gen_ids.push_back(all_ids[i]); }
   }
   const mape_extract_args* const* items = gen.data();
