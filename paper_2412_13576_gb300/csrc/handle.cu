@@ -212,7 +212,10 @@ struct mape_instance {
       }
     }
     cudaMemPool_t pool = library_pool(dev);
-    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, stream) != cudaSuccess) return nullptr;
+    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, stream) != cudaSuccess) {
+      cudaGetLastError();  // the launches that follow do not see it
+      return nullptr;
+    }
     return p;
   }
   void release(void* p, size_t bytes) {
@@ -237,7 +240,8 @@ struct mape_instance {
   // allocation may be a call into the caller's allocator (the Python binding's
   // takes the interpreter's lock, tens of microseconds each, one thread at a
   // time): a handle's 33 allocations and as many releases were most of the time of 16
-  // requests at once, 57 ms; 28 with one per stage.
+  // requests at once, 57 ms; 28 with one per stage.  An allocator that has no
+  // block of that size left is asked for the buffers one by one.
   struct Buffers {
     std::vector<std::pair<size_t, std::function<void(char*)>>> parts;
     size_t bytes = 0;
@@ -248,9 +252,16 @@ struct mape_instance {
       bytes += mape_detail::align_up(std::max<size_t>(16, count * sizeof(T)), 256);
     }
     bool place(mape_instance* h, std::vector<std::pair<void*, size_t>>& list) {
-      char* base = h->take<char>(list, bytes);
-      if (!base) return false;
-      for (auto& part : parts) part.second(base + part.first);
+      if (char* base = h->take<char>(list, bytes)) {
+        for (auto& part : parts) part.second(base + part.first);
+        return true;
+      }
+      for (size_t k = 0; k < parts.size(); ++k) {
+        const size_t end = k + 1 < parts.size() ? parts[k + 1].first : bytes;
+        char* at = h->take<char>(list, end - parts[k].first);
+        if (!at) return false;
+        parts[k].second(at);
+      }
       return true;
     }
   };
