@@ -366,6 +366,7 @@ __device__ __forceinline__ void stream_fwd_body(const StParams& p, const int blk
     for (int ch = h; ch < N / 16; ch += 2) {
       uint32_t v[16];
       if (fwd) {
+        __syncwarp();  // the loads and their waits are for a converged warp
         tmem_ld16(tmem + lane_base + ch * 16, v);
         tc_wait_ld();
         uint32_t w[8];
@@ -381,6 +382,7 @@ __device__ __forceinline__ void stream_fwd_body(const StParams& p, const int blk
         *reinterpret_cast<uint4*>(Sp + chunk_off(r, kg % kKC + 8)) = make_uint4(w[4], w[5], w[6], w[7]);
       }
       if (collect) {
+        __syncwarp();
         tmem_ld16(tmem + lane_base + p.wF + ch * 16, v);
         tc_wait_ld();
         const int i0 = row0 + ch * 16;
@@ -744,6 +746,7 @@ __device__ __forceinline__ void stream_grad_body(const StParams& p, const int bl
       float4 nz[2] = {cz[0], cz[1]}, nm[2] = {cm[0], cm[1]}, nv[2] = {cv[0], cv[1]};
       if (ch + 2 < nch) load_state(ch + 2, nz, nm, nv);
       uint32_t gv[8];
+      __syncwarp();  // converged for the load and its wait
       tmem_ld8(tmem + lane_base + ch * 8, gv);
       float zc[8] = {cz[0].x, cz[0].y, cz[0].z, cz[0].w, cz[1].x, cz[1].y, cz[1].z, cz[1].w};
       float mc[8] = {cm[0].x, cm[0].y, cm[0].z, cm[0].w, cm[1].x, cm[1].y, cm[1].z, cm[1].w};

@@ -483,6 +483,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
     bool out = false;
     for (int ch = split; ch < nch; ch += kSplits) {
       uint32_t v[8];
+      __syncwarp();
       tmem_ld8x2(tmem + lane_off + colD2 + ch * 16, v);
       tc_wait_ld();
 #pragma unroll
@@ -573,6 +574,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
       // rows of B' from D2 (warp-collective loads: every lane executes them)
       for (int ch = split; ch < nch; ch += kSplits) {
         uint32_t v[8];
+        __syncwarp();  // lanes without a slot have skipped what came before
         tmem_ld8x2(tmem + lane_off + colD2 + ch * 16, v);
         tc_wait_ld();
 #pragma unroll
@@ -586,6 +588,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
     } else {
       for (int ch = split; ch < nch; ch += kSplits) {
         uint32_t v[8];
+        __syncwarp();  // lanes without a slot have skipped what came before
         tmem_ld8x2(tmem + lane_off + colD2 + ch * 16, v);
         tc_wait_ld();
         uint32_t w[2] = {0, 0};
@@ -695,6 +698,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
       if (!late) test_candidate();
     }
     if (collect_prev && tid == 0) *s_any = 0;  // every thread read it in the last write_candidate
+    __syncwarp();
     tc_wait_ld();
     tc_fence_before();
     fence_async_smem();
@@ -796,6 +800,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
       const int c0 = ub + W * half;
       uint32_t v[W];
       float zc[W], mc[W], vc[W], rz[W], g[W];
+      __syncwarp();  // the lanes wrote their outputs one by one
       load_state(ub, c0, v, zc, mc, vc);
 #pragma unroll
       for (int c = 0; c < W; ++c) rz[c] = rintf(zc[c]);
@@ -815,6 +820,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
         if (u < nu16) dbg_unit(Width<8>{}, 16 * u);
         else dbg_unit(Width<4>{}, 16 * nu16 + 8 * (u - nu16));
       }
+      __syncwarp();
     }
     float nzinf = 0.f;
     int nkmax = kNoNz, first_id = kNoNz;
@@ -946,6 +952,7 @@ __device__ __forceinline__ void extract_tc_body(const TcParams& p, const int til
       test_candidate();
     }
     if (tid == 0) *s_any = 0;
+    __syncwarp();
     tc_wait_ld();
     if (__syncthreads_or(late)) {
       if (tid == 0) atomicOr(p.flags, 16);
