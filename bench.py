@@ -601,11 +601,11 @@ def kernel_case(args):
 
 
 def streamed_case(args):
-    """The streamed kernels (three per step) alone on a named instance, with
-    the large workload's starts and collection period: per step, the forward
-    pass reads z (4 d bytes per start) and writes sign(Bm z) (2 R bytes), the
-    gradient pass reads it back and reads and writes z, m, v (24 d bytes): the
-    algorithmic bytes are 28 d + 4 R per start-step."""
+    """The streamed extraction alone on a named instance, with the large
+    workload's starts and collection period.  A step reads and writes the
+    state z, m, v of a start once: 24 d algorithmic bytes.  The step-by-step
+    kernels (three per step: a sparse forward pass) read z once more, 4 d
+    bytes, and write and read sign(Bm z), 2 R bytes each: 28 d + 4 R."""
     import torch
     from paper_2412_13576_gb300 import instances as I
     from paper_2412_13576_gb300 import mape
@@ -626,7 +626,7 @@ def streamed_case(args):
                                         period=LARGE["period"])
     ms = statistics.median(times)
     R = inst.n - inst.d
-    algo = (28.0 * inst.d + 4.0 * R) * P * T
+    algo = (28.0 * inst.d + 4.0 * R if args.sparse_fwd else 24.0 * inst.d) * P * T
     peaks, src = measured_peaks()
     gbs = algo / (ms / 1e3) / 1e9
     return {"streamed_case": {"instance": inst.name, "n": inst.n, "d": inst.d, "P": P, "T": T,
@@ -865,7 +865,7 @@ def batch_pipeline_measure(N, T=1000, seed=1003):
 
 
 RESIDENT_TRAFFIC = os.path.join(ROOT, "profiles", "extract_tc_kernel_medium_sparse_P8192_T1000_traffic.md")
-STREAM_TRAFFIC = os.path.join(ROOT, "profiles", "stream_step_large_quartic_traffic.md")
+STREAM_TRAFFIC = os.path.join(ROOT, "profiles", "cluster_kernel_large_quartic_traffic.md")
 
 
 def measured_traffic(record, src_path):
@@ -888,10 +888,10 @@ def measured_traffic(record, src_path):
 def roofline_streamed(mape, wl, inst, starts, stream, prec, reps=2):
     """The streamed extraction of the large workload, timed live: `reps` calls
     of mape_extract (T steps, the workload's starts and period).  A step reads
-    and writes the FP32 state z, m, v of every start and moves its operands of
-    z and signs; counted as (28 d + 4 R) P bytes (the state once in and out, z
-    once more, sign(Bm z) out and in) over the step's time (the call's time
-    over T, which includes turning z, m, v once per call).  The bound is HBM
+    and writes the FP32 state z, m, v of every start once, 24 d P bytes, over
+    the step's time (the call's time over T, which includes turning z, m, v
+    once per call); of the operands and signs, which the blocks of a tile pass
+    on through L2, a part reaches HBM and is not counted.  The bound is HBM
     bandwidth: the state (1.26 GB) is far larger than L2 and is streamed every
     step.  Beside it, the launches of the step-by-step kernels (those of a
     general B, which launch timing makes every call run)."""
@@ -910,7 +910,7 @@ def roofline_streamed(mape, wl, inst, starts, stream, prec, reps=2):
     peak = peaks["hbm_gbs"]
     call_ms = statistics.median(times)
     step_ms = call_ms / T
-    step_bytes = (28.0 * d + 4.0 * R) * P
+    step_bytes = 24.0 * d * P  # the FP32 state once each way
     achieved = step_bytes / (step_ms / 1e3) / 1e9
     kernels = {}
     for kind, name, per_start in (("stream_grad", "stream_grad_kernel", 24.0 * d + 2.0 * R),
@@ -930,9 +930,9 @@ def roofline_streamed(mape, wl, inst, starts, stream, prec, reps=2):
             "step_by_step": {"ms_per_step": statistics.median(stepwise) / T, "kernels": kernels},
             "collect_ms_per_launch": per["stream_collect"][0] / max(per["stream_collect"][1], 1),
             "candidates_per_call": int(np.median(counts)),
-            "note": "one step = forward + gradient (+ collection every period-th step) for P = 65536 starts, 28 d + 4 R "
-                    "bytes per start; step time = CUDA-event time of a T = 1000 call / T (the call also packs z, m, v "
-                    "once); step_by_step: the kernels that launch timing makes the call run, from events the library "
+            "note": "one step = forward + gradient (+ collection every period-th step) for P = 65536 starts, 24 d "
+                    "bytes per start (z, m, v in FP32 read and written once); step time = CUDA-event time of a T = 1000 call "
+                    "/ T (the call also packs z, m, v once); step_by_step: the kernels that launch timing makes the call run, from events the library "
                     "records around each launch; traffic = ncu dram read+write bytes of one step, null unless taken "
                     "on this source"}
 

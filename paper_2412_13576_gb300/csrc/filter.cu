@@ -1112,7 +1112,8 @@ extern "C" int mape_kernel_test_batch(mape_kernel_test_item* items, int32_t coun
     it.fail_count = 0;
     KtView& d = v[(size_t)i];
     d = KtView{it.A, it.m, it.n, it.ldg, it.G, it.K, it.ok, nullptr, nullptr, nullptr, nullptr};
-    // the compressed rows in the instance's own workspace, carved as mape_kernel_test carves it
+    // the compressed rows in the instance's own workspace (of mape_kernel_test_workspace_bytes; one word in
+    // front where the single call takes two, which round up alike)
     Carver cv(it.workspace, it.workspace_bytes);
     cv.take<unsigned long long>(1);
     d.rowcnt = cv.take<uint32_t>((size_t)it.m + 1);

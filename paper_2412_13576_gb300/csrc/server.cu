@@ -236,7 +236,9 @@ void mape_server::start_batch(std::vector<Request*>& rs) {
   cv.notify_all();
 }
 
-// Called with the lock held: releases the request's slot and memory.
+// Called with the lock held: releases the request's slot and memory (and waits
+// for the handle's buffers to go back and for its slot's stream, which has
+// finished its work).
 void mape_server::finish(Request* r, int err) {
   if (r->h) {
     mape_destroy(r->h);
