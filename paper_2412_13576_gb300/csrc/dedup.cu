@@ -189,7 +189,7 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;  // consecutive pairs of a thread
 constexpr int kSortTile = kSortThreads * kSortItems;
 
-// Where the merge of A (na sorted pairs) and B (nb) has given `diag` pairs:
+// Merge path (Green, Odeh and Birk): where the merge of A (na sorted pairs) and B (nb) has given `diag` pairs:
 // how many of them come from A (from A first among equals).  ka/ia/kb/ib read
 // a pair.
 template <typename KA, typename IA, typename KB, typename IB>
